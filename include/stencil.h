@@ -115,9 +115,10 @@ typedef struct {
                          not 16-byte multiples run on the tensor-core kernels through two
                          padded grids the plan owns (one strided copy in, one out per apply) */
     int32_t unit_planes; /* 3D matrixized kernel: output planes per work unit, 1..1024 (0 = the
-                         library's 32).  Each unit streams its planes plus 2r halo planes, so
-                         the depth trades re-read halo planes against the number of units
-                         (load balance); exposed for the scheduling ablation          */
+                         library's choice by the grid's size, up to 32).  Each unit streams
+                         its planes plus 2r halo planes, so the depth trades re-read halo
+                         planes against the number of units (load balance); exposed for the
+                         scheduling ablation                                            */
     int32_t reserved[1];
 } stencil_options;
 

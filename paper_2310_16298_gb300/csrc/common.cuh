@@ -41,6 +41,30 @@ cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, fn, std::forward<A>(args)...);
 }
 
+// Planes per work unit of a 3D sweep: units are `tiles` columns cut into
+// ceil(nz / c) chunks, processed by `slots` workers at about (c + fixed) plane
+// times each (`fixed`: halo planes and pipeline fill).  Returns the c <= most
+// with the shortest estimated sweep; the deeper of equals, which re-reads
+// fewer halo planes.  A fixed depth (64 planes, tensor cores 32) left small
+// grids on a few SMs and large ones with a nearly empty last wave; us per
+// sweep before and after: FP64 star 64^3 328 / 11, 512^3 1982 / 1956; FP32
+// gather 27-point 128^3 81 / 11, 512^3 375 / 336; tensor cores (with columns
+// of one quarter each, below) 27-point 64^3 29 / 8.6, 256^3 78 / 52,
+// 512^3 416 / 359, 7-point 512^3 229 / 200.
+inline int pick_chunk(int nz, int64_t tiles, int64_t slots, int fixed, int most) {
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int c = 1; c <= most && c <= nz; ++c) {
+        const int64_t units = tiles * ((nz + c - 1) / c);
+        const int64_t cost = (units + slots - 1) / slots * (c + fixed);
+        if (cost <= best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 __host__ __device__ inline int64_t wrap_index(int64_t i, int64_t n) {
     int64_t m = i % n;
     return m < 0 ? m + n : m;

@@ -636,13 +636,13 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
     }
 }
 
-// 3D streaming kernel: a work unit is TZC output planes of a TY x TX column;
-// its TZC + 2R input planes stream through NPL = 2R + 2 plane buffers.
+// 3D streaming kernel: a work unit is a.tzc output planes of a TY x TX column
+// (chosen per grid by pick_chunk); its tzc + 2R input planes stream through
+// NPL = 2R + 2 plane buffers.
 template <typename T>
 struct Tile3 {
     static constexpr int TY = 32;
     static constexpr int TX = 64;
-    static constexpr int TZC = 64;
     static constexpr int AL = 16 / (int)sizeof(T);
 };
 constexpr int kThreads3 = 256;   // (TY / kRS) strips x TX columns
@@ -653,7 +653,8 @@ struct G3Args {
     unsigned int* err;
     int64_t ldx;         // row stride of the grids (elements); planes are ny rows
     int nz, ny, nx, bc;
-    int tiles_x, tiles_y, chunks, units;
+    int tiles_x, tiles_y, units;
+    int tzc;             // output planes per work unit
 };
 
 template <typename T, int R>
@@ -670,7 +671,7 @@ template <typename T, int R, bool STAR>
 __global__ void __launch_bounds__(kThreads3, min_ctas<T, 3>())
 gather3d_stream_kernel(const __grid_constant__ CUtensorMap tin, const G3Args a, const Coeffs<T, ipow(2 * R + 1, 3)> cf) {
     using L = Layout3<T, R>;
-    constexpr int W = 2 * R + 1, TY = Tile3<T>::TY, TX = Tile3<T>::TX, TZC = Tile3<T>::TZC, NPL = L::NPL;
+    constexpr int W = 2 * R + 1, TY = Tile3<T>::TY, TX = Tile3<T>::TX, NPL = L::NPL;
     static_assert(TX * (TY / kRS) == kThreads3, "one strip per thread");
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char* smem_raw = (unsigned char*)(((uintptr_t)smem_dyn + 127) & ~(uintptr_t)127);
@@ -695,8 +696,8 @@ gather3d_stream_kernel(const __grid_constant__ CUtensorMap tin, const G3Args a, 
     unsigned int in_flight = 0;          // buffers with a TMA load nobody waited for yet (bit mask)
     for (int u = blockIdx.x; u < a.units && !*abort_flag; u += gridDim.x) {
         const int tx_ = u % a.tiles_x, ty_ = (u / a.tiles_x) % a.tiles_y, tz_ = u / (a.tiles_x * a.tiles_y);
-        const int x0 = tx_ * TX, y0 = ty_ * TY, z0 = tz_ * TZC;
-        const int nout = min(TZC, a.nz - z0);
+        const int x0 = tx_ * TX, y0 = ty_ * TY, z0 = tz_ * a.tzc;
+        const int nout = min(a.tzc, a.nz - z0);
         // with a periodic boundary, an edge unit's planes (staged by TMA like
         // the others, from the wrapped plane index) get their cells outside
         // the grid in y and x wrapped once they have landed
@@ -939,8 +940,6 @@ cudaError_t launch3d(const GatherProblem& p, const void* in, void* out, int tb, 
     a.bc = p.bc;
     a.tiles_x = (a.nx + Tile3<T>::TX - 1) / Tile3<T>::TX;
     a.tiles_y = (a.ny + Tile3<T>::TY - 1) / Tile3<T>::TY;
-    a.chunks = (a.nz + Tile3<T>::TZC - 1) / Tile3<T>::TZC;
-    a.units = a.tiles_x * a.tiles_y * a.chunks;
     alignas(64) CUtensorMap tin;
     const cuuint64_t dims[3] = {(cuuint64_t)a.nx, (cuuint64_t)a.ny, (cuuint64_t)a.nz};
     const cuuint32_t box[3] = {(cuuint32_t)L::SX, (cuuint32_t)L::SY, 1};
@@ -952,6 +951,12 @@ cudaError_t launch3d(const GatherProblem& p, const void* in, void* out, int tb, 
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads3, smem);
     if (e != cudaSuccess) return e;
     int grid = sm_count() * (per > 0 ? per : 1);
+    // A unit's fixed cost in planes: FP32 units re-read 2R halo planes and wait
+    // for the first 2R + 1 to land; FP64 units compute far longer than that per
+    // plane.
+    const int tiles = a.tiles_x * a.tiles_y;
+    a.tzc = pick_chunk(a.nz, tiles, grid, sizeof(T) == 8 ? 1 : 2 * R + 2, 64);
+    a.units = tiles * ((a.nz + a.tzc - 1) / a.tzc);
     if (grid > a.units) grid = a.units;
     kern<<<grid, kThreads3, smem, s>>>(tin, a, cf);
     return cudaGetLastError();

@@ -13,8 +13,11 @@
 // z - (a - R).  When input plane z has been scattered, output plane z - R is
 // complete and is written with one TMA store.
 //
-// Work unit = (32-row-slab tile in y, NB columns in x, a chunk of output
-// planes in z); the unit streams its chunk plus R halo planes on either side.
+// Work unit = four columns (a quarter of 32 input rows in y, NB columns in x;
+// one per lane quarter) and a chunk of output planes in z; the unit streams
+// its chunk plus R halo planes on either side.  The quarters take columns in
+// running order, x fastest, instead of four y quarters of one x tile: 512 rows
+// are 18 quarters of 30, not 20, so a 512^3 sweep computes a tenth less.
 // Boundaries: the zero Dirichlet halo is TMA's out-of-bounds fill; with a
 // periodic boundary the producer wraps the plane index (whole planes), and the
 // terms that wrap in x or y are added afterwards by the edge kernel
@@ -53,7 +56,11 @@ constexpr int kMaxRawStages = 6;
 constexpr int kUnitRing = 8;                // unit ids handed from the producer to the epilogue
 constexpr int kTmemCols = 512;
 constexpr int kSmemBudget = 227 * 1024;
-constexpr int kChunk = 32;  // output planes per work unit (library choice; plans may set their own)
+// Deepest work unit the library chooses (plans may set their own depth): at 512^3
+// 16 to 32 planes ran fastest, 64 and 128 slower (fewer units to balance).
+constexpr int kMaxChunk = 32;
+// Pipeline fill and drain of a unit, in plane times (pick_chunk's fixed cost beside the 2R halo planes).
+constexpr int kFillPlanes = 2;
 
 // Coefficient lines of a 3D stencil: (a = z offset, b = y offset) pairs that
 // carry weights.  Box: all (2R+1)^2 pairs.  Star, parallel cover: (a, R) for
@@ -118,7 +125,9 @@ struct MxArgs3D {
     int nz, ny, nx;
     int64_t ldx;          // row stride of the grids (elements); planes are ny rows
     int nparts;           // operand parts of the input split (1..3)
-    int tiles_x, tiles_y, chunks, units;
+    int tiles_x;          // x tiles (NB columns)
+    int groups;           // units per chunk: the (y quarter, x tile) columns in fours
+    int units;
     int chunk;            // output planes per work unit
     uint32_t bop_bytes;
     uint32_t bpart_bytes;
@@ -148,7 +157,6 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
     constexpr int RSB = raw_stage_bytes3(KP);
     constexpr int kRawStages = raw_stages3(NB, LM, BF);
     constexpr int OWB = out_warp_bytes3(NB);
-    const int PLANES = args.chunk + 2 * R;  // input planes per work unit
     constexpr uint32_t SLAB_BOX = (uint32_t)(kSlabRows * KP * 4);
     static_assert(kRawStages >= 3, "TMA ring too shallow");
     static_assert(N <= 256 && N % 16 == 0, "MMA N");
@@ -216,11 +224,18 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
     const uint32_t tmem_d = tmem + (uint32_t)(AST * A_COLS);
     int issued = 0, committed = -1;
 
-    // unit u -> (x tile, y tile, z chunk), x fastest
-    auto unit_origin = [&](int u, int& X0, int& Y0, int& Z0) {
-        X0 = (u % args.tiles_x) * NB;
-        Y0 = ((u / args.tiles_x) % args.tiles_y) * (kQuarters * ROWS_OUT);
-        Z0 = (u / (args.tiles_x * args.tiles_y)) * args.chunk;
+    // Unit u: z chunk u / groups (the last one may be shorter) of the columns
+    // 4 g .. 4 g + 3, g = u % groups; column c is x tile c % tiles_x of the y
+    // quarter (ROWS_OUT rows) c / tiles_x, one per lane quarter.  Columns past
+    // the last lie below the grid: zeros are loaded and nothing is stored.
+    auto unit_planes = [&](int u, int& Z0) {   // input planes of the unit
+        Z0 = (u / args.groups) * args.chunk;
+        return min(args.chunk, args.nz - Z0) + 2 * R;
+    };
+    auto column = [&](int u, int q, int& X0, int& Y0) {
+        const int c = (u % args.groups) * kQuarters + q;
+        X0 = (c % args.tiles_x) * NB;
+        Y0 = (c / args.tiles_x) * ROWS_OUT;
     };
 
     if (warp == 0) {
@@ -246,9 +261,11 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
                     }
                     break;
                 }
-                int X0, Y0, Z0;
-                unit_origin(u, X0, Y0, Z0);
-                for (int iz = 0; iz < PLANES; ++iz, ++i) {
+                int X0[kQuarters], Y0[kQuarters], Z0;
+#pragma unroll
+                for (int q = 0; q < kQuarters; ++q) column(u, q, X0[q], Y0[q]);
+                const int planes = unit_planes(u, Z0);
+                for (int iz = 0; iz < planes; ++iz, ++i) {
                     const int s = i % kRawStages;
                     const uint32_t ph = (uint32_t)(i / kRawStages) & 1u;
                     if (!wait_or_abort(&rawfree[s], ph ^ 1u, abort_flag)) {
@@ -262,8 +279,7 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
                     ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)kQuarters * SLAB_BOX);
 #pragma unroll
                     for (int q = 0; q < kQuarters; ++q)
-                        ptx::tma_load_3d(dst + q * SLAB_BOX, &tmap, X0 - kPad, Y0 + q * ROWS_OUT - R, gz,
-                                         &full[s]);
+                        ptx::tma_load_3d(dst + q * SLAB_BOX, &tmap, X0[q] - kPad, Y0[q] - R, gz, &full[s]);
                     issued = i + 1;
                 }
             }
@@ -360,13 +376,14 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
                 if (lane == 0) ptx::mbar_arrive(&uq_empty[uq]);
                 if (u < 0) break;
                 int X0, Y0, Z0;
-                unit_origin(u, X0, Y0, Z0);
+                column(u, q, X0, Y0);
+                const int planes = unit_planes(u, Z0);
                 float acc[2 * R + 1][CW];  // running sums of output planes z-R .. z+R
 #pragma unroll
                 for (int j = 0; j < 2 * R + 1; ++j)
 #pragma unroll
                     for (int c = 0; c < CW; ++c) acc[j][c] = 0.0f;
-                for (int iz = 0; iz < PLANES; ++iz, ++i) {
+                for (int iz = 0; iz < planes; ++iz, ++i) {
                     const int st = i % DST;
                     const uint32_t ph = (uint32_t)(i / DST) & 1u;
                     if (!wait_or_abort(&accf[st], ph, abort_flag)) {
@@ -473,9 +490,9 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
                         }
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
-                        const int ox = X0 + CW * sub, oy = Y0 + q * ROWS_OUT;
-                        if (lane == 0 && ox < args.nx && oy < args.ny && Z0 + iz - 2 * R < args.nz) {
-                            ptx::tma_store_3d(&tmap_out, ox, oy, Z0 + iz - 2 * R, ost);
+                        const int ox = X0 + CW * sub;
+                        if (lane == 0 && ox < args.nx && Y0 < args.ny) {
+                            ptx::tma_store_3d(&tmap_out, ox, Y0, Z0 + iz - 2 * R, ost);
                             ptx::bulk_commit_group();
                         }
                         ++nstore;
@@ -732,7 +749,7 @@ cudaError_t mx3d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     const Mx3State* st = (const Mx3State*)p.tmap_storage;
     const int nz = (int)p.n[0], ny = (int)p.n[1], nx = (int)p.n[2];
     const int in_w = st->in_w;
-    const int rows_tile = kQuarters * (kSlabRows - 2 * p.r);
+    const int rows_out = kSlabRows - 2 * p.r;   // output rows per y quarter
     MxArgs3D a;
     memset(&a, 0, sizeof(a));
     a.bc = p.bc;
@@ -747,10 +764,9 @@ cudaError_t mx3d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     a.nprod = products_for(p.prec);
     a.bpart_bytes = st->bpart_bytes;
     a.tiles_x = (nx + st->nb - 1) / st->nb;
-    a.tiles_y = (ny + rows_tile - 1) / rows_tile;
-    a.chunk = p.unit_planes > 0 ? p.unit_planes : kChunk;
-    a.chunks = (nz + a.chunk - 1) / a.chunk;
-    a.units = a.tiles_x * a.tiles_y * a.chunks;
+    a.groups = (a.tiles_x * ((ny + rows_out - 1) / rows_out) + kQuarters - 1) / kQuarters;
+    a.chunk = p.unit_planes > 0 ? p.unit_planes : pick_chunk(nz, a.groups, st->num_sms, 2 * p.r + kFillPlanes, kMaxChunk);
+    a.units = a.groups * ((nz + a.chunk - 1) / a.chunk);
     a.bop_bytes = st->bop_bytes;
     alignas(64) CUtensorMap map, map_out;
     if (!encode_in_map_3d(&map, (const float*)src, nz, ny, nx, p.ldx, raw_pitch3(in_w))) return cudaErrorInvalidValue;
