@@ -107,7 +107,11 @@ typedef struct {
     int32_t prec;     /* stencil_precision; default NATIVE for GATHER, TF32X3 for F32 MATRIXIZED */
     int32_t bc;       /* stencil_boundary; default DIRICHLET_ZERO                              */
     int32_t impl;     /* stencil_impl; default AUTO                                            */
-    int32_t tb;       /* time steps fused per sweep (temporal blocking); 0 = library choice     */
+    int32_t tb;       /* time steps fused per sweep (temporal blocking); 0 = library choice: 1,
+                         or, for 2D matrixized plans of order 1 / 2 in TF32X3 or BF16X3 with
+                         extents of at least 96, up to 4 / 2 steps evaluated as one step of
+                         the composed stencil.  An apply of n steps then runs n / tb whole
+                         sweeps and a shorter last one                                       */
     int32_t cover;    /* stencil_cover; default AUTO (EINVAL when out of range)                 */
     int32_t pitch;    /* row stride of the grids, in elements (0 = packed rows); >= the
                          contiguous extent and a multiple of 16 bytes, else EINVAL.  Padding
@@ -135,7 +139,8 @@ typedef struct {
                              bounded wait (or stencil_plan_raise_error set bits)        */
     int32_t cover;        /* stencil_cover the matrixized kernel runs (0 for GATHER)    */
     int32_t kernels_per_sweep; /* kernel launches per sweep: 2 for MATRIXIZED plans with
-                             a periodic boundary (the tensor-core kernel, whose TMA
+                             a periodic boundary, except 2D ones of FP32-class
+                             arithmetic with extents of at least 96 (the tensor-core kernel, whose TMA
                              loads see zeros outside the grid in x and y, then a
                              kernel over the boundary strips that adds the wrapped
                              terms), else 1                                             */
@@ -321,7 +326,7 @@ STENCIL_API stencil_status stencil_batch_run(int n, const stencil_plan_t *plans,
  * plus 1 MiB: its own grid, advanced in place, and its plan's scratch grid,
  * the second copy of the ping-pong) and the resident-slot
  * limit allow.  Every resident request advances by at most `quantum_steps`
- * time steps per issue on one of `nstreams` streams, so requests overlap on
+ * time steps (whole sweeps of its plan, at least one) per issue on one of `nstreams` streams, so requests overlap on
  * the device and new ones join as soon as memory and a slot free up.  A
  * finished grid is copied to host memory and the request's device state is
  * freed.  Each request runs through the same plan and kernels as

@@ -64,6 +64,7 @@
 #include <cudaTypedefs.h>
 #include <string.h>
 
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <type_traits>
@@ -90,8 +91,14 @@ constexpr int kTw = kItems * kNb;       // output columns per tile
 constexpr int kSplitWarps = 2 * kQuarters;   // (quarter, input row parity)
 constexpr int kEpiWarps = 2 * kQuarters;     // (quarter, output row parity)
 constexpr int kMma2Warp = 2 + kSplitWarps + kEpiWarps;   // second MMA issuer
-constexpr int kThreads = 32 * (kMma2Warp + 1);
-constexpr int kBopCopies = 16;          // copies of the banded operands in global memory
+constexpr int kStripWarp = kMma2Warp + 1;                // boundary strips
+constexpr int kThreads = 32 * (kStripWarp + 1);
+constexpr int kMaxDepth = 4;            // time steps one sweep can advance
+constexpr int kStripMin = 96;           // smallest extent of a grid whose boundary strips run in the sweep's kernel
+constexpr int kStripCols = 4;           // columns of the left strip: one 16-byte group
+constexpr int kStripRow = 12;           // floats per row of a strip weight table (2R+1 weights, 16-byte rows)
+constexpr int kBopCopies = 16;          // most copies of the banded operands in global memory
+constexpr int kCtasPerCopy = 10;        // CTAs that read one copy when a sweep starts
 constexpr int kMaxRawStages = 6;
 constexpr int kTileRing = 8;            // tile ids handed from the producer to the epilogue
 constexpr int kTmemCols = 512;
@@ -149,12 +156,19 @@ __host__ __device__ constexpr int smem_bytes() {
 struct MxArgs2D {
     const void* bops;          // block operands [part][kchunk][block*16 + q][16 bytes]
     unsigned int* err;         // device error word (host-mapped)
-    int* sched;                // [0] next tile to hand out, [1] CTAs finished (both 0 between launches)
+    int* sched;                // [0] tiles handed out beyond the first gridDim.x, [1] CTAs finished (0 between launches)
     int ny, nx;
     int64_t ldx;               // row stride of the grids (elements)
     int nparts;                // operand parts of the input split (1..3)
     int tiles_x, tiles_total;
-    int rows_even, rows_odd;   // rows of the even / odd row-parity views
+    int x0, y0, x1, y1;        // grid region the tiles write: rows y0.., columns x0..; the rest are strips
+    int rows_even, rows_odd;   // that region's rows of the even / odd row-parity views
+    int bc;
+    int strip_classes;         // weight classes per axis of the strips (0: no strips)
+    const float* strip_w;      // strip weights [y class][x class][2R+1][kStripRow]
+    const float* in;
+    float* out;
+    int bop_copies;
     uint32_t bop_bytes;        // every part
     uint32_t bpart_bytes;      // one part
     int nprod;                 // products per K step (1, 3 or 6)
@@ -170,6 +184,113 @@ __host__ __device__ constexpr int d_sets(int a_cols, int n) {
     return (a_stages(a_cols, n) * a_cols + 4 * n <= kTmemCols)   ? 4
            : (a_stages(a_cols, n) * a_cols + 3 * n <= kTmemCols) ? 3
                                                                  : 2;
+}
+
+// Boundary strips.  The points within a few rows or columns of a face are not
+// a convolution with one set of weights: with a zero halo, a sweep of k > 1
+// steps resets the points outside the grid after every step, so the weights
+// depend on the distance to the faces; with a periodic boundary the neighbours
+// wrap, which the tiles' TMA loads (zeros outside the grid) do not.  One warp
+// per CTA computes them from global memory in FP32 beside the tiles: an item
+// is four adjacent columns of one row, the weights come from a table by the
+// point's distance class in y and x (one class when periodic).  The tiles
+// write only the rest of the grid, so the two need no order between them.
+// 8192^2, order 4: 32 thousand items over 152 warps cost 8 us of a 134 us
+// sweep (issue slots and the load/store pipe shared with the tiles' warps); a
+// second kernel over the strips cost 20.  Data comes through L2 (__ldcg): the
+// buffer was the output of an earlier sweep of the same stream.
+__device__ __forceinline__ int strip_class(int i, int n, int s) {
+    return i < s ? i : (n - 1 - i < s ? 2 * s - (n - 1 - i) : s);
+}
+
+template <int R>
+__device__ __forceinline__ void boundary_strips(const MxArgs2D& a, int first, int stride) {
+    constexpr int W = 2 * R + 1;
+    constexpr int RB = 3;                     // input rows loaded before the first is used
+    const int groups = (a.nx + 3) >> 2;       // column groups per row
+    const int xg = a.x1 >> 2;                 // first group right of the tiles' region
+    const int left = a.x0 >> 2;               // groups left of the tiles' region
+    const int side = left + groups - xg;      // strip groups of a row beside it
+    const int mid = a.y1 - a.y0;
+    const int full = (a.y0 + a.ny - a.y1) * groups;   // items of whole rows
+    const int total = full + mid * side;
+    const int s = a.strip_classes >> 1;
+    const bool periodic = a.bc == kBcPeriodic;
+    for (int item = first; item < total; item += stride) {
+        int y, g;
+        if (item < full) {
+            const int f = item / groups;
+            g = item - f * groups;
+            y = f < a.y0 ? f : a.y1 + (f - a.y0);
+        } else {   // consecutive lanes: consecutive rows of one group
+            const int j = item - full, c = j / mid;
+            y = a.y0 + j - c * mid;
+            g = c < left ? c : xg + c - left;
+        }
+        const float* wy = a.strip_w + (size_t)strip_class(y, a.ny, s) * a.strip_classes * (W * kStripRow);
+        int cx[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cx[q] = strip_class(min(4 * g + q, a.nx - 1), a.nx, s);
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int d0 = 0; d0 < W; d0 += RB) {
+            float v[RB][12];   // v[b][k] = column 4 g - 4 + k of row y - R + d0 + b
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                int yy = y - R + d0 + b;
+                const bool wrap_y = yy < 0 || yy >= a.ny;
+                const bool use = d0 + b < W && (periodic || !wrap_y);
+                if (wrap_y) yy += yy < 0 ? a.ny : -a.ny;
+                const float* row = a.in + (int64_t)yy * a.ldx;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int x = 4 * (g - 1 + k);
+                    float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (use && x >= 0 && x + 3 < a.nx) {
+                        u = __ldcg(reinterpret_cast<const float4*>(row + x));
+                    } else if (use) {   // group across the x face: column by column
+                        auto at = [&](int c) {
+                            if (c >= 0 && c < a.nx) return __ldcg(row + c);
+                            return periodic ? __ldcg(row + (c < 0 ? c + a.nx : c - a.nx)) : 0.0f;
+                        };
+                        u = make_float4(at(x), at(x + 1), at(x + 2), at(x + 3));
+                    }
+                    v[b][4 * k] = u.x;
+                    v[b][4 * k + 1] = u.y;
+                    v[b][4 * k + 2] = u.z;
+                    v[b][4 * k + 3] = u.w;
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                if (d0 + b >= W) break;
+                float w[kStripRow];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q == 0 || cx[q] != cx[q - 1]) {
+                        const float* wr = wy + ((size_t)cx[q] * W + d0 + b) * kStripRow;
+#pragma unroll
+                        for (int c = 0; c < (W + 3) / 4; ++c) {
+                            const float4 u = __ldg(reinterpret_cast<const float4*>(wr) + c);
+                            w[4 * c] = u.x;
+                            w[4 * c + 1] = u.y;
+                            w[4 * c + 2] = u.z;
+                            w[4 * c + 3] = u.w;
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < W; ++c) acc[q] = fmaf(w[c], v[b][4 + q + c - R], acc[q]);
+                }
+            }
+        }
+        float* o = a.out + (int64_t)y * a.ldx + 4 * g;
+        if (4 * g + 3 < a.nx) {
+            *reinterpret_cast<float4*>(o) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (4 * g + q < a.nx) o[q] = acc[q];
+        }
+    }
 }
 
 template <int R, bool BF, int NP>
@@ -248,6 +369,10 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
         *abort_flag = 0;
         ptx::fence_mbar_init();
     }
+    const bool claims = (int)gridDim.x < args.tiles_total;   // more tiles than CTAs
+    // A small grid lets the stream's next kernel start at once: on the SMs that
+    // this one leaves free its CTAs set themselves up and wait.
+    if (!claims && tid == 32 * kStripWarp) ptx::launch_dependents();
     if (warp == 1) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
         ptx::tmem_relinquish();
@@ -265,13 +390,19 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
             ptx::mbar_arrive_expect_tx(bop_bar, args.bop_bytes);
-            ptx::bulk_load(bops, (const unsigned char*)args.bops + (size_t)(blockIdx.x % kBopCopies) * args.bop_bytes,
+            ptx::bulk_load(bops, (const unsigned char*)args.bops + (size_t)(blockIdx.x % args.bop_copies) * args.bop_bytes,
                            args.bop_bytes, bop_bar);
+            ptx::prefetch_tensormap(&tmap_e);
+            ptx::prefetch_tensormap(&tmap_o);
+            ptx::prefetch_tensormap(&omap_e);
+            ptx::prefetch_tensormap(&omap_o);
             // Launched as a programmatic dependent of the stream's previous
             // kernel (the previous sweep, or its boundary-strip kernel): the
             // set-up above (barriers, tensor memory, banded operands) overlapped
             // its tail; the grids and the tile counter are touched only from here.
             ptx::grid_dependency_wait();
+            // A CTA's first tile is its index: no claim to wait for, and none at
+            // all on a grid with a CTA per tile.
             for (int i = 0;; ++i) {
                 const int s = i % kRawStages;
                 const uint32_t ph = (uint32_t)(i / kRawStages) & 1u;
@@ -279,7 +410,8 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                 if (!wait_or_abort(&rawfree[s], ph ^ 1u, abort_flag) ||
                     !wait_or_abort(&tq_empty[tq], ((uint32_t)(i / kTileRing) & 1u) ^ 1u, abort_flag))
                     break;
-                int t = atomicAdd(&args.sched[0], 1);
+                int t = blockIdx.x;
+                if (i > 0) t = claims ? (int)gridDim.x + atomicAdd(&args.sched[0], 1) : args.tiles_total;
                 if (t >= args.tiles_total) t = -1;
                 stage_tile[s] = t;
                 tile_ring[tq] = t;
@@ -288,8 +420,8 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                     ptx::mbar_arrive(&full[s]);
                     break;
                 }
-                const int X0 = (t % args.tiles_x) * kTw;
-                const int Y0 = (t / args.tiles_x) * (kQuarters * G::ROWS_OUT);
+                const int X0 = args.x0 + (t % args.tiles_x) * kTw;
+                const int Y0 = args.y0 + (t / args.tiles_x) * (kQuarters * G::ROWS_OUT);
                 unsigned char* dst = raw + s * RSB;
                 ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)RSB);
 #pragma unroll
@@ -383,6 +515,17 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                 if (lane == 0) ptx::mbar_arrive(&afull[sa]);
             }
         }
+    } else if (warp == kStripWarp) {
+        // ------------------------------------------------ boundary strips (straight from and to global memory)
+        if (args.strip_classes > 0) {
+            // bring the weights (at most 21 KB) into L1 while the previous kernel
+            // drains: read cold, row by row, they were most of a small grid's sweep
+            constexpr int kTable = (2 * R + 1) * kStripRow;
+            for (int o = lane * 32; o < args.strip_classes * args.strip_classes * kTable; o += 32 * 32)
+                ptx::prefetch_l1(args.strip_w + o);
+            ptx::grid_dependency_wait();
+            boundary_strips<R>(args, blockIdx.x * 32 + lane, gridDim.x * 32);
+        }
     } else {
         // ------------------------------------------------ epilogue: accumulators -> outputs (warps 10..17)
         const int q = warp & 3;
@@ -413,7 +556,7 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                     break;
                 }
                 ptx::tc_fence_after();
-                const int X0 = (t % args.tiles_x) * kTw;
+                const int X0 = (t % args.tiles_x) * kTw;   // in the tiles' region
                 const int Y0 = (t / args.tiles_x) * (kQuarters * G::ROWS_OUT);
                 const uint32_t dbase = tmem_d + lane_off + (uint32_t)(st * N + P * G::NBP * kNb);
                 float acc[kNb];
@@ -485,7 +628,7 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                     ptx::fence_proxy_async_smem();
                     __syncwarp();
                     const int oy = (Y0 + q * G::ROWS_OUT) / 2;   // first output row of the quarter, parity view
-                    if (lane == 0 && X0 < args.nx && oy < prows) {
+                    if (lane == 0 && X0 < args.x1 - args.x0 && oy < prows) {
                         ptx::tma_store_2d(omap, X0, oy, ost);
                         ptx::bulk_commit_group();
                     }
@@ -517,7 +660,8 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
     if (tid == 0 && *abort_flag) atomicOr(args.err, 1u);
     ptx::tc_fence_before();
     __syncthreads();
-    if (tid == 0) {   // every producer of this CTA is done: the last CTA resets the tile counter
+    // every producer of this CTA is done: the last CTA resets the tile counter
+    if (tid == 0 && claims) {
         __threadfence();
         if (atomicAdd(&args.sched[1], 1) == (int)gridDim.x - 1) {
             atomicExch(&args.sched[0], 0);
@@ -594,15 +738,120 @@ bool encode_parity_map(CUtensorMap* map, const float* base, int rows_p, int nx, 
                CU_TENSOR_MAP_INTERLEAVE_NONE, swz, l2, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// What a sweep of one depth needs (offsets into the plan's operand buffer).
+struct DepthOps {
+    int order = 0;             // order of the composed stencil, depth * r
+    size_t bops = 0;           // banded operands
+    int copies = 1;            // of the banded operands, one after the other
+    uint32_t bop_bytes = 0;
+    uint32_t bpart_bytes = 0;
+    int strip_rows = 0;        // rows (columns) along each face computed as strips (0: none)
+    int strip_classes = 0;
+    size_t strip_w = 0;
+};
+
 struct MxState {
     unsigned int* err_host = nullptr;  // host-mapped error word
     unsigned int* err_dev = nullptr;
-    int* sched = nullptr;              // device tile counter pair (zero between launches)
+    int* sched = nullptr;              // device tile counter pair (in the operand buffer; zero between launches)
     int num_sms = 0;
     bool bf = false;      // BF16 operands (else TF32)
-    uint32_t bop_bytes = 0;
-    uint32_t bpart_bytes = 0;
+    DepthOps depth[kMaxDepth + 1];     // [1 .. the plan's tb]
 };
+
+constexpr size_t kSchedBytes = 256;    // of the operand buffer: the tile counters
+
+// Tiles of a region of ny x nx outputs for a stencil of order r.
+int64_t tiles_2d(int64_t ny, int64_t nx, int r) {
+    const int rows = kQuarters * 2 * (kLanes - 2 * ((r + 1) / 2));
+    return (nx + kTw - 1) / kTw * ((ny + rows - 1) / rows);
+}
+
+// Weights of `k` steps of a 2D stencil as one stencil of order k r: what the
+// input at each offset contributes to one output point when the points past
+// the given limits (offsets from the output point) are outside the grid, that
+// is, zero at every step in between.  Without limits this is the k-fold
+// convolution of the weights.
+struct Limits {
+    int ylo, yhi, xlo, xhi;
+};
+constexpr int kNoLimit = 1 << 20;
+
+std::vector<double> compose_steps(int r, const double* cg, int k, const Limits& in) {
+    const int R = k * r, W = 2 * R + 1, w = 2 * r + 1;
+    std::vector<double> cur((size_t)W * W, 0.0), nxt;
+    cur[(size_t)R * W + R] = 1.0;
+    for (int step = 1; step <= k; ++step) {
+        nxt.assign(cur.size(), 0.0);
+        const int h = (step - 1) * r;
+        for (int y = -h; y <= h; ++y)
+            for (int x = -h; x <= h; ++x) {
+                const double v = cur[(size_t)(y + R) * W + x + R];
+                if (v == 0.0) continue;
+                for (int a = 0; a < w; ++a)
+                    for (int b = 0; b < w; ++b) {
+                        const int yy = y + a - r, xx = x + b - r;
+                        if (yy < in.ylo || yy > in.yhi || xx < in.xlo || xx > in.xhi) continue;
+                        nxt[(size_t)(yy + R) * W + xx + R] += cg[a * w + b] * v;
+                    }
+            }
+        cur.swap(nxt);
+    }
+    return cur;
+}
+
+// Split precisions that stand in for FP32 arithmetic; only these fuse steps.
+// In the others the rounding of the weights and of the field at every step is
+// part of the result a caller asked for.
+bool fp32_class(int prec) { return prec == STENCIL_PREC_TF32X3 || prec == STENCIL_PREC_BF16X3; }
+
+bool strips_in_kernel(const MxRequest& q) {
+    return fp32_class(q.prec) && q.n[0] >= kStripMin && q.n[1] >= kStripMin;
+}
+
+// Time steps per sweep.  k steps of an order-r stencil are one step of an
+// order-kr stencil, and the sweep's time grows far slower than k: 8192^2 TF32x3,
+// us per sweep for order 1 / 2 / 3 / 4: 89 / 94 / 113 / 125, so as many steps
+// as the largest order built (4) holds: 4 steps of order 1 in 125 us instead
+// of 356, 2 of order 2 instead of 188.  Only when the composed weights are as
+// safe as the single steps: within FP32's range by a wide margin, and with no
+// larger a rounding error (the composed weights' absolute sum bounds it; k
+// single steps have k times the weights' absolute sum, times the growth of a
+// constant field).
+int fused_depth(const MxRequest& q) {
+    if (q.tb != 0 || !strips_in_kernel(q)) return 1;
+    const int w = 2 * q.r + 1;
+    double sum = 0.0, abs_sum = 0.0;
+    for (int i = 0; i < w * w; ++i) {
+        sum += q.cg[i];
+        abs_sum += std::fabs(q.cg[i]);
+    }
+    if (!(abs_sum > std::ldexp(1.0, -24) && abs_sum < std::ldexp(1.0, 24))) return 1;
+    for (int k = std::min(kMaxDepth, 4 / q.r); k > 1; --k) {
+        double composed = 0.0;
+        for (double v : compose_steps(q.r, q.cg, k, {-kNoLimit, kNoLimit, -kNoLimit, kNoLimit})) composed += std::fabs(v);
+        if (composed <= 1.0001 * k * abs_sum * std::max(1.0, std::pow(std::fabs(sum), k - 1))) return k;
+    }
+    return 1;
+}
+
+// Strip weights of depth k: [y class][x class][2R+1][kStripRow], classes 0 ..
+// s-1 by the distance to the low face, s past both, s+1 .. 2s up to the high
+// face (s = (k-1) r for the zero halo, 0 when periodic).
+std::vector<float> strip_weights(int r, const double* cg, int k, int s) {
+    const int R = k * r, W = 2 * R + 1, n = 2 * s + 1;
+    std::vector<float> out((size_t)n * n * W * kStripRow, 0.0f);
+    auto lo = [&](int c) { return c < s ? -c : -kNoLimit; };
+    auto hi = [&](int c) { return c > s ? 2 * s - c : kNoLimit; };
+    for (int cy = 0; cy < n; ++cy)
+        for (int cx = 0; cx < n; ++cx) {
+            const std::vector<double> c = compose_steps(r, cg, k, {lo(cy), hi(cy), lo(cx), hi(cx)});
+            for (int a = 0; a < W; ++a)
+                for (int b = 0; b < W; ++b)
+                    out[(((size_t)cy * n + cx) * W + a) * kStripRow + b] = (float)c[(size_t)a * W + b];
+        }
+    return out;
+}
 
 }  // namespace
 
@@ -664,27 +913,61 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
     const bool bf = is_bf16(q.prec);
     const int W = bf ? window<true>(kNb) : window<false>(kNb);
     p->nb = kNb;
-    const auto blocks = pair_blocks(q.r, q.cg);
-    uint32_t bpart = 0;
-    std::vector<unsigned char> ops = pack_blocks(q.r, blocks, kNb, W, bf, &bpart);
+    p->tb = fused_depth(q);
     p->n_lines = 2 * q.r + 1;
     p->cover = STENCIL_COVER_PARALLEL;
     p->n_scalar = 0;
-    const size_t one = ops.size();   // one copy; CTA b reads copy b % kBopCopies
-    p->operand_bytes = one * kBopCopies;
-    const KernelInfo ki = kernel_for(q.r, bf, operand_parts(q.prec));
-    if (!ki.fn || one != (size_t)(bf ? 3 : 2) * bpart || one % 16 != 0) {
-        if (why) *why = "internal error: block operand size";
-        return STENCIL_EUNSUPPORTED;
+    // One buffer: the tile counter pair (zero), each depth's strip weights and
+    // banded operands, the whole sweeps' operands last and in several copies
+    // (CTA b reads copy b % copies).
+    DepthOps depth[kMaxDepth + 1];
+    std::vector<unsigned char> all(kSchedBytes, 0);
+    const bool strips = strips_in_kernel(q);
+    for (int k = 1; k <= p->tb; ++k) {
+        DepthOps& d = depth[k];
+        d.order = k * q.r;
+        d.strip_rows = !strips ? 0 : q.bc == kBcPeriodic ? d.order : (k - 1) * q.r;
+        if (d.strip_rows > 0) {
+            const int s = q.bc == kBcPeriodic ? 0 : d.strip_rows;
+            const std::vector<float> w = strip_weights(q.r, q.cg, k, s);
+            d.strip_classes = 2 * s + 1;
+            d.strip_w = all.size();
+            all.insert(all.end(), (const unsigned char*)w.data(), (const unsigned char*)(w.data() + w.size()));
+        }
+        const std::vector<double> cg = compose_steps(q.r, q.cg, k, {-kNoLimit, kNoLimit, -kNoLimit, kNoLimit});
+        const std::vector<unsigned char> ops = pack_blocks(d.order, pair_blocks(d.order, cg.data()), kNb, W, bf,
+                                                           q.prec == STENCIL_PREC_TF32X3 && p->tb > 1, &d.bpart_bytes);
+        d.bop_bytes = (uint32_t)ops.size();
+        if (!kernel_for(d.order, bf, operand_parts(q.prec)).fn || d.bop_bytes != (bf ? 3 : 2) * d.bpart_bytes ||
+            d.bop_bytes % 16 != 0) {
+            if (why) *why = "internal error: block operand size";
+            return STENCIL_EUNSUPPORTED;
+        }
+        d.bops = all.size();
+        all.insert(all.end(), ops.begin(), ops.end());
     }
-    std::vector<unsigned char> copies(p->operand_bytes);
-    for (int c = 0; c < kBopCopies; ++c) memcpy(copies.data() + c * one, ops.data(), one);
-    cudaError_t e = cudaMalloc(&p->d_operands, p->operand_bytes);
+    DepthOps& last = depth[p->tb];
+    int dev = 0, num_sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t ctas = std::min<int64_t>(num_sms, tiles_2d(q.n[0], q.n[1], last.order));
+    last.copies = (int)std::min<int64_t>(kBopCopies, (ctas + kCtasPerCopy - 1) / kCtasPerCopy);
+    p->operand_bytes = all.size() + (size_t)(last.copies - 1) * last.bop_bytes;
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_operands, p->operand_bytes);
     if (e != cudaSuccess) {
+        p->d_operands = nullptr;
         if (why) *why = std::string("operand upload: ") + cudaGetErrorString(e);
         return STENCIL_ENOMEM;
     }
-    e = cudaMemcpy(p->d_operands, copies.data(), p->operand_bytes, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(p->d_operands, all.data(), all.size(), cudaMemcpyHostToDevice);
+    unsigned char* const first = (unsigned char*)p->d_operands + last.bops;
+    for (int have = 1; have < last.copies && e == cudaSuccess;) {   // 1 -> 2 -> 4 .. copies
+        const int more = std::min(have, last.copies - have);
+        e = cudaMemcpyAsync(first + (size_t)have * last.bop_bytes, first, (size_t)more * last.bop_bytes,
+                            cudaMemcpyDeviceToDevice, cudaStreamLegacy);
+        have += more;
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         cudaFree(p->d_operands);
         p->d_operands = nullptr;
@@ -692,8 +975,7 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
         return STENCIL_ECUDA;
     }
     MxState* st = new MxState();
-    st->bop_bytes = (uint32_t)one;
-    st->bpart_bytes = bpart;
+    for (int k = 1; k <= p->tb; ++k) st->depth[k] = depth[k];
     st->bf = bf;
     e = cudaHostAlloc((void**)&st->err_host, sizeof(unsigned int), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&st->err_dev, st->err_host, 0);
@@ -705,24 +987,19 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
         return STENCIL_ECUDA;
     }
     *st->err_host = 0;
+    st->sched = (int*)p->d_operands;
+    st->num_sms = num_sms;
     p->tmap_storage = st;
-    e = cudaMalloc(&st->sched, 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(st->sched, 0, 2 * sizeof(int));
-    if (e != cudaSuccess) {
-        mx_plan_free(p);
-        if (why) *why = std::string("tile counter: ") + cudaGetErrorString(e);
-        return STENCIL_ENOMEM;
+    for (int k = 1; k <= p->tb && e == cudaSuccess; ++k) {
+        const KernelInfo ki = kernel_for(k * q.r, bf, operand_parts(q.prec));
+        e = cudaFuncSetAttribute(ki.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ki.smem);
     }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    e = cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ki.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ki.smem);
     if (e != cudaSuccess) {
         mx_plan_free(p);
         if (why) *why = std::string("kernel set-up: ") + cudaGetErrorString(e);
         return STENCIL_ECUDA;
     }
-    return with_edges(q, p, why);
+    return strips ? STENCIL_OK : with_edges(q, p, why);   // the strips cover the periodic boundary
 }
 
 void mx_plan_free(MxPlan* p) {
@@ -735,7 +1012,6 @@ void mx_plan_free(MxPlan* p) {
     MxState* st = (MxState*)p->tmap_storage;
     if (st) {
         if (st->err_host) cudaFreeHost(st->err_host);
-        if (st->sched) cudaFree(st->sched);
         delete st;
     }
     p->tmap_storage = nullptr;
@@ -754,16 +1030,16 @@ cudaError_t mx_sweep(const MxPlan& p, const void* src, void* dst, int tb, cudaSt
 }
 
 cudaError_t mx2d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cudaStream_t s) {
-    if (tb != 1) return cudaErrorInvalidValue;
+    if (tb < 1 || tb > p.tb) return cudaErrorInvalidValue;
     if (((uintptr_t)src & 15u) || ((uintptr_t)dst & 15u)) return cudaErrorMisalignedAddress;
     const MxState* st = (const MxState*)p.tmap_storage;
+    const DepthOps& d = st->depth[tb];
     const int ny = (int)p.n[0], nx = (int)p.n[1];
-    const int dm = (p.r + 1) / 2;
-    const int rows_out = 2 * (kLanes - 2 * dm);          // output rows per quarter
+    const int dm = (d.order + 1) / 2;
     const int RWD = st->bf ? raw_row<true>(kNb) : raw_row<false>(kNb);
     MxArgs2D a;
     memset(&a, 0, sizeof(a));
-    a.bops = p.d_operands;
+    a.bops = (const unsigned char*)p.d_operands + d.bops;
     a.err = st->err_dev;
     a.sched = st->sched;
     a.ny = ny;
@@ -771,28 +1047,49 @@ cudaError_t mx2d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     a.ldx = p.ldx;
     a.nparts = operand_parts(p.prec);
     a.nprod = products_for(p.prec);
-    a.bpart_bytes = st->bpart_bytes;
-    a.tiles_x = (nx + kTw - 1) / kTw;
-    a.tiles_total = a.tiles_x * ((ny + kQuarters * rows_out - 1) / (kQuarters * rows_out));
-    a.rows_even = (ny + 1) / 2;
-    a.rows_odd = ny / 2;
-    a.bop_bytes = st->bop_bytes;
-    const float* in = (const float*)src;
-    float* out = (float*)dst;
+    a.bpart_bytes = d.bpart_bytes;
+    a.bop_bytes = d.bop_bytes;
+    a.bop_copies = d.copies;
+    a.bc = p.bc;
+    a.in = (const float*)src;
+    a.out = (float*)dst;
+    // The tiles' region: all of the grid, or what the strips leave, from an even
+    // row (row-parity views) and a whole 32-byte sector.
+    a.x1 = nx;
+    a.y1 = ny;
+    int64_t items = 0;
+    if (d.strip_rows > 0) {
+        a.strip_classes = d.strip_classes;
+        a.strip_w = (const float*)((const unsigned char*)p.d_operands + d.strip_w);
+        a.x0 = kStripCols;
+        a.y0 = (d.strip_rows + 1) / 2 * 2;
+        a.x1 = (nx - d.strip_rows) / 4 * 4;
+        a.y1 = ny - d.strip_rows;
+        const int groups = (nx + 3) / 4;
+        items = (int64_t)(a.y0 + ny - a.y1) * groups + (int64_t)(a.y1 - a.y0) * (a.x0 / 4 + groups - a.x1 / 4);
+    }
+    const int rx = a.x1 - a.x0, ry = a.y1 - a.y0;
+    a.tiles_x = (rx + kTw - 1) / kTw;
+    a.tiles_total = (int)tiles_2d(ry, rx, d.order);
+    a.rows_even = (ry + 1) / 2;
+    a.rows_odd = ry / 2;
+    const int64_t ld = p.ldx;
+    float* const out = a.out + a.y0 * ld + a.x0;
     alignas(64) CUtensorMap te, to, oe, oo;
     const int kp = raw_pitch(RWD);
-    const int64_t ld = p.ldx;
-    if (!encode_parity_map(&te, in, a.rows_even, nx, ld, kp, kLanes, CU_TENSOR_MAP_SWIZZLE_NONE,
+    if (!encode_parity_map(&te, a.in, (ny + 1) / 2, nx, ld, kp, kLanes, CU_TENSOR_MAP_SWIZZLE_NONE,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B) ||
-        !encode_parity_map(&to, in + ld, a.rows_odd, nx, ld, kp, kLanes, CU_TENSOR_MAP_SWIZZLE_NONE,
+        !encode_parity_map(&to, a.in + ld, ny / 2, nx, ld, kp, kLanes, CU_TENSOR_MAP_SWIZZLE_NONE,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B) ||
-        !encode_parity_map(&oe, out, a.rows_even, nx, ld, kTw, kLanes - 2 * dm, CU_TENSOR_MAP_SWIZZLE_128B,
+        !encode_parity_map(&oe, out, a.rows_even, rx, ld, kTw, kLanes - 2 * dm, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_NONE) ||
-        !encode_parity_map(&oo, out + ld, a.rows_odd, nx, ld, kTw, kLanes - 2 * dm, CU_TENSOR_MAP_SWIZZLE_128B,
+        !encode_parity_map(&oo, out + ld, a.rows_odd, rx, ld, kTw, kLanes - 2 * dm, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_NONE))
         return cudaErrorInvalidValue;
-    const KernelInfo ki = kernel_for(p.r, st->bf, operand_parts(p.prec));
-    const int grid = a.tiles_total < st->num_sms ? a.tiles_total : st->num_sms;
+    const KernelInfo ki = kernel_for(d.order, st->bf, operand_parts(p.prec));
+    // a CTA per tile or per warp of strip items, up to one per SM
+    const int64_t want = std::max<int64_t>(a.tiles_total, (items + 31) / 32);
+    const int grid = (int)std::min<int64_t>(want, st->num_sms);
     return launch_dependent(ki.fn, grid, kThreads, ki.smem, s, te, to, oe, oo, a);
 }
 

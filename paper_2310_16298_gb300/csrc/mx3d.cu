@@ -121,7 +121,7 @@ struct MxArgs3D {
     int bc;               // periodic: input planes wrap in z (x and y: edges.cu)
     const void* bops;     // banded operands [part][kchunk][line*NB + q][16 bytes]
     unsigned int* err;    // device error word (host-mapped)
-    int* sched;           // [0] next unit to hand out, [1] CTAs finished (both 0 between launches)
+    int* sched;           // [0] units handed out beyond the first gridDim.x, [1] CTAs finished (0 between launches)
     int nz, ny, nx;
     int64_t ldx;          // row stride of the grids (elements); planes are ny rows
     int nparts;           // operand parts of the input split (1..3)
@@ -212,6 +212,8 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
         *abort_flag = 0;
         ptx::fence_mbar_init();
     }
+    const bool claims = (int)gridDim.x < args.units;   // more units than CTAs
+    if (!claims && tid == 32 * kMma2Warp) ptx::launch_dependents();   // small grids, as in the 2D kernel
     if (warp == 1) {
         ptx::tmem_alloc(tmem_slot, kTmemCols);
         ptx::tmem_relinquish();
@@ -242,6 +244,8 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
         if (lane == 0) {
             ptx::mbar_arrive_expect_tx(bop_bar, args.bop_bytes);
             ptx::bulk_load(bops, args.bops, args.bop_bytes, bop_bar);
+            ptx::prefetch_tensormap(&tmap);
+            ptx::prefetch_tensormap(&tmap_out);
             // programmatic dependent launch: grids and the unit counter only from here
             ptx::grid_dependency_wait();
             int i = 0;
@@ -249,7 +253,8 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
             for (int k = 0; ok; ++k) {
                 const int uq = k % kUnitRing;
                 if (!wait_or_abort(&uq_empty[uq], ((uint32_t)(k / kUnitRing) & 1u) ^ 1u, abort_flag)) break;
-                int u = atomicAdd(&args.sched[0], 1);
+                int u = blockIdx.x;   // the first unit; the others are claimed
+                if (k > 0) u = claims ? (int)gridDim.x + atomicAdd(&args.sched[0], 1) : args.units;
                 if (u >= args.units) u = -1;
                 unit_ring[uq] = u;
                 ptx::mbar_arrive(&uq_full[uq]);
@@ -524,7 +529,8 @@ mx3d_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CU
     if (tid == 0 && *abort_flag) atomicOr(args.err, 1u);
     ptx::tc_fence_before();
     __syncthreads();
-    if (tid == 0) {   // this CTA's producer is done: the last CTA resets the unit counter
+    // this CTA's producer is done: the last CTA resets the unit counter
+    if (tid == 0 && claims) {
         __threadfence();
         if (atomicAdd(&args.sched[1], 1) == (int)gridDim.x - 1) {
             atomicExch(&args.sched[0], 0);

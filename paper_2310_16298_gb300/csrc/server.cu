@@ -234,7 +234,10 @@ void worker_loop(stencil_server_s* S) {
             }
             cudaStream_t s = S->streams[q->stream];
             if (q->done_steps < q->steps) {
-                const int64_t k = std::min<int64_t>(S->quantum, q->steps - q->done_steps);
+                // whole sweeps (a plan may advance several steps per sweep), so that
+                // the steps fuse as in one apply of all of them
+                const int64_t tb = q->plan->tb;
+                const int64_t k = std::min<int64_t>(std::max<int64_t>(S->quantum / tb, 1) * tb, q->steps - q->done_steps);
                 stencil_status st = stencil_apply(q->plan, q->grid, q->grid, k, (stencil_stream_t)s);
                 if (st != STENCIL_OK) {
                     q->error = st;
