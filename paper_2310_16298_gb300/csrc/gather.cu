@@ -47,6 +47,11 @@ __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
 
+__device__ __forceinline__ void cp_async_16(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Address of a tile element after the boundary rule, or nullptr for a zero.
@@ -71,6 +76,191 @@ __device__ __forceinline__ const T* src3(const T* __restrict__ a, int64_t z, int
         x = wrap_index(x, nx);
     }
     return a + (z * ny + y) * ldx + x;
+}
+
+// ---------------------------------------------------------------------------
+// 2D FP32 sub-steps, register-blocked: a thread computes kVR rows x 4 adjacent
+// columns.  Each input row it needs is read as three 16-byte shared-memory
+// loads (columns x-4 .. x+7, enough for r <= 4) and every weight is applied to
+// four columns at once, so an update costs its P FMAs and about one
+// shared-memory load (the scalar strips spend about 7.5 loads and the index
+// arithmetic around them).  The sum of an output runs over the rows, then the
+// columns of C^g in order, as everywhere in this file: results do not depend
+// on tiles, depth or blocking.
+// ---------------------------------------------------------------------------
+constexpr int kVR = 4;         // rows per thread
+constexpr int kSlackRows = 4;  // rows after a buffer that ragged blocks read (and, before the last sub-step, write)
+
+// base = element (row of the first output - R, column of the first output - 4).
+template <int R, bool STAR>
+__device__ __forceinline__ void block_f32(const float* base, int SX, const Coeffs<float, ipow(2 * R + 1, 2)>& cf,
+                                          float (&acc)[kVR][4]) {
+    static_assert(R <= 4, "three 16-byte loads cover x-4 .. x+7");
+    constexpr int W = 2 * R + 1;
+#pragma unroll
+    for (int j = 0; j < kVR; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+#pragma unroll
+    for (int yi = 0; yi < kVR + 2 * R; ++yi) {
+        float v[12];   // v[k] = column x - 4 + k of input row yi
+#pragma unroll
+        for (int k4 = 0; k4 < 3; ++k4) {
+            const float4 u = *reinterpret_cast<const float4*>(base + yi * SX + 4 * k4);
+            v[4 * k4] = u.x;
+            v[4 * k4 + 1] = u.y;
+            v[4 * k4 + 2] = u.z;
+            v[4 * k4 + 3] = u.w;
+        }
+#pragma unroll
+        for (int j = 0; j < kVR; ++j) {
+            const int a = yi - j;
+            if (a >= 0 && a < W) {
+#pragma unroll
+                for (int b = 0; b < W; ++b)
+                    if (!STAR || a == R || b == R) {
+                        const float w = cf.c[a * W + b];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) acc[j][q] = fmaf(w, v[4 + q + b - R], acc[j][q]);
+                    }
+            }
+        }
+    }
+}
+
+// Geometry of a tile of TY x TX outputs in shared memory for depth tb: H halo
+// rows, HX halo columns (a multiple of 4), SY x SX elements.  Element (sy, sx)
+// is grid point (y0 - H + sy, x0 - HX + sx).
+struct TileGeom {
+    int H, HX, SY, SX;
+    __host__ __device__ TileGeom(int r, int tb, int ty, int tx)
+        : H(r * tb), HX((r * tb + 3) / 4 * 4), SY(ty + 2 * r * tb), SX(tx + 2 * ((r * tb + 3) / 4 * 4)) {}
+    // One buffer: the tile, then the slack rows (which also end the last row's ragged reads).
+    __host__ __device__ int elems() const { return (SY + kSlackRows) * SX; }
+};
+constexpr int kLeadElems = 32;   // before the first buffer: ragged reads left of row 0
+
+// Sub-step t < tb of a tile: src -> dst, both in shared memory.  Rows R t ..
+// SY - R t and the columns that the later sub-steps still need are computed,
+// rounded out to whole blocks: the extra cells read cells outside the tile
+// (neighbouring rows' ends, slack), hold garbage and are never used.  `zero`
+// (tiles across the grid's edge, zero boundary): cells outside the grid are
+// zero again after the sub-step.
+template <int R, bool STAR, int TX>
+__device__ __forceinline__ void substep_f32(const float* src, float* dst, const TileGeom& g, int t, int tb, bool zero,
+                                            int ny, int nx, int gy0, int gx0, int tid, int nthreads,
+                                            const Coeffs<float, ipow(2 * R + 1, 2)>& cf) {
+    const int lo = R * t;
+    const int c0 = (g.HX - R * (tb - t)) & ~3;
+    const int ncg = (g.HX + TX + R * (tb - t) - c0 + 3) >> 2;
+    const int nstrips = (g.SY - 2 * lo + kVR - 1) / kVR;
+    const unsigned magic = ((1u << 20) + ncg - 1) / ncg;   // item / ncg = item * magic >> 20 for items below 2^20 / ncg
+    for (int item = tid; item < nstrips * ncg; item += nthreads) {
+        const int strip = (int)((item * magic) >> 20), cgi = item - strip * ncg;
+        const int sy = lo + strip * kVR, sx = c0 + 4 * cgi;
+        float acc[kVR][4];
+        block_f32<R, STAR>(src + (sy - R) * g.SX + (sx - 4), g.SX, cf, acc);
+        if (zero) {
+#pragma unroll
+            for (int j = 0; j < kVR; ++j) {
+                const int gy = gy0 + sy + j;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int gx = gx0 + sx + q;
+                    if (gy < 0 || gy >= ny || gx < 0 || gx >= nx) acc[j][q] = 0.0f;
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kVR; ++j)
+            *reinterpret_cast<float4*>(dst + (sy + j) * g.SX + sx) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+    }
+}
+
+// Last sub-step of a tile, to the grid: the valid region starts at the aligned
+// column HX, so rows of four outputs go out as 16-byte stores when the grid's
+// rows are 16-byte aligned (`vec`).
+template <int R, bool STAR, int TY, int TX>
+__device__ __forceinline__ void last_substep_f32(const float* src, float* __restrict__ out, const TileGeom& g, bool vec,
+                                                 int ny, int nx, int64_t ldx, int y0, int x0, int tid, int nthreads,
+                                                 const Coeffs<float, ipow(2 * R + 1, 2)>& cf) {
+    static_assert(TY % kVR == 0 && TX % 4 == 0, "whole blocks");
+    constexpr int ncg = TX / 4;
+    for (int item = tid; item < TY / kVR * ncg; item += nthreads) {
+        const int strip = item / ncg, cgi = item - strip * ncg;   // a warp: consecutive column groups
+        float acc[kVR][4];
+        block_f32<R, STAR>(src + (g.H + strip * kVR - R) * g.SX + (g.HX + 4 * cgi - 4), g.SX, cf, acc);
+        const int gx = x0 + 4 * cgi;
+#pragma unroll
+        for (int j = 0; j < kVR; ++j) {
+            const int gy = y0 + strip * kVR + j;
+            if (gy < ny) {
+                float* o = out + (int64_t)gy * ldx + gx;
+                if (vec && gx + 3 < nx) {
+                    *reinterpret_cast<float4*>(o) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (gx + q < nx) o[q] = acc[j][q];
+                }
+            }
+        }
+    }
+}
+
+// One FP32 tile (origin y0, x0) loaded element by element (any row alignment,
+// either boundary) and advanced by tb steps; buffers a and b ping-pong.  A
+// grid without 16-byte rows gets its outputs through shared memory: written
+// as blocks, four 4-byte stores 16 bytes apart per lane would touch every
+// sector four times.
+template <int R, bool STAR, int TY, int TX>
+__device__ __forceinline__ void tile2_f32(const float* __restrict__ in, float* __restrict__ out, int ny, int nx,
+                                          int64_t ldx, int bc, int tb, const Coeffs<float, ipow(2 * R + 1, 2)>& cf,
+                                          int y0, int x0, float* a, float* b, int tid, int nthreads) {
+    const TileGeom g(R, tb, TY, TX);
+    const int gy0 = y0 - g.H, gx0 = x0 - g.HX;
+    const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
+    const bool inside = gy0 >= 0 && gy0 + g.SY <= ny && gx0 >= 0 && gx0 + g.SX <= nx;
+    const bool vec = ldx % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+    for (int sy = warp; sy < g.SY; sy += nwarps) {
+        float* d = a + sy * g.SX;
+        if (inside && vec) {
+            const float* s = in + (int64_t)(gy0 + sy) * ldx + gx0;
+            for (int sx = 4 * lane; sx < g.SX; sx += 128) cp_async_16(d + sx, s + sx);
+        } else if (inside) {
+            const float* s = in + (int64_t)(gy0 + sy) * ldx + gx0;
+            for (int sx = lane; sx < g.SX; sx += 32) cp_async_elem(d + sx, s + sx);
+        } else {
+            for (int sx = lane; sx < g.SX; sx += 32) {
+                const float* s = src2(in, gy0 + sy, gx0 + sx, ny, nx, ldx, bc);
+                if (s) cp_async_elem(d + sx, s);
+                else d[sx] = 0.0f;
+            }
+        }
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    const bool zero = !inside && bc == kBcDirichlet;
+    for (int t = 1; t < tb; ++t) {
+        substep_f32<R, STAR, TX>(a, b, g, t, tb, zero, ny, nx, gy0, gx0, tid, nthreads, cf);
+        float* const other = a;
+        a = b;
+        b = other;
+        __syncthreads();
+    }
+    if (vec) {
+        last_substep_f32<R, STAR, TY, TX>(a, out, g, true, ny, nx, ldx, y0, x0, tid, nthreads, cf);
+    } else {
+        substep_f32<R, STAR, TX>(a, b, g, tb, tb, false, ny, nx, gy0, gx0, tid, nthreads, cf);
+        __syncthreads();
+        const int cols = min(TX, nx - x0);
+        for (int y = warp; y < TY && y0 + y < ny; y += nwarps) {
+            const float* s = b + (g.H + y) * g.SX + g.HX;
+            float* o = out + (int64_t)(y0 + y) * ldx + x0;
+            for (int x = lane; x < cols; x += 32) o[x] = s[x];
+        }
+    }
+    __syncthreads();   // both buffers are free
 }
 
 // ---------------------------------------------------------------------------
@@ -162,34 +352,52 @@ __global__ void __launch_bounds__(kBX * BY)
 gather2d_kernel(const T* __restrict__ in, T* __restrict__ out, int64_t ny, int64_t nx, int64_t ldx, int bc,
                 int tb, Coeffs<T, ipow(2 * R + 1, 2)> cf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    gather2d_tile<T, R, STAR, BY, TX, TY>(in, out, ny, nx, ldx, bc, tb, cf, (int64_t)blockIdx.y * TY,
-                                          (int64_t)blockIdx.x * TX, reinterpret_cast<T*>(smem_raw));
+    if constexpr (sizeof(T) == 4) {
+        float* a = reinterpret_cast<float*>(smem_raw) + kLeadElems;
+        tile2_f32<R, STAR, TY, TX>(in, out, (int)ny, (int)nx, ldx, bc, tb, cf, (int)blockIdx.y * TY, (int)blockIdx.x * TX,
+                                   a, a + TileGeom(R, tb, TY, TX).elems(), threadIdx.y * kBX + threadIdx.x, kBX * BY);
+    } else {
+        gather2d_tile<T, R, STAR, BY, TX, TY>(in, out, ny, nx, ldx, bc, tb, cf, (int64_t)blockIdx.y * TY,
+                                              (int64_t)blockIdx.x * TX, reinterpret_cast<T*>(smem_raw));
+    }
 }
 
 // Persistent batched sweep: the tiles of many independent problems, each
 // advanced by its own depth, processed by one grid-stride launch.  Problem
 // p owns tiles [tile0[p], tile0[p+1]); its coefficients sit at coef + p*NC.
 template <typename T, int R, bool STAR, int BY, int TX, int TY>
-__global__ void __launch_bounds__(kBX * BY)
+__global__ void __launch_bounds__(kBX * BY, sizeof(T) == 4 && R == 1 ? 16 / BY + 1 : 1)
 gather2d_batch_kernel(const BatchProblem* __restrict__ probs, int nprob, int total_tiles,
                       const T* __restrict__ coef) {
     constexpr int NC = ipow(2 * R + 1, 2);
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    int lo = 0;   // problem of tile t: the last one whose first tile <= t
     for (int t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-        int lo = 0, hi = nprob - 1;  // last problem whose first tile <= t
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (probs[mid].tile0 <= t) lo = mid;
-            else hi = mid - 1;
+        // a CTA's tiles ascend: search on from the previous tile's problem, a
+        // warp's width at a time (each lane one candidate)
+        for (;;) {
+            const int k = lo + 1 + (int)threadIdx.x;
+            const unsigned past = __ballot_sync(0xffffffffu, k >= nprob || probs[k].tile0 > t);
+            if (past) {
+                lo += __ffs(past) - 1;
+                break;
+            }
+            lo += 32;
         }
         const BatchProblem P = probs[lo];
         const int local = t - P.tile0;
+        const int y0 = local / P.tiles_x * TY, x0 = local % P.tiles_x * TX;
         Coeffs<T, NC> cf;
 #pragma unroll
         for (int i = 0; i < NC; ++i) cf.c[i] = coef[(size_t)P.coef_index * NC + i];
-        gather2d_tile<T, R, STAR, BY, TX, TY>((const T*)P.src, (T*)P.dst, P.ny, P.nx, P.nx, P.bc, P.depth, cf,
-                                              (int64_t)(local / P.tiles_x) * TY, (int64_t)(local % P.tiles_x) * TX,
-                                              reinterpret_cast<T*>(smem_raw));
+        if constexpr (sizeof(T) == 4) {
+            float* a = reinterpret_cast<float*>(smem_raw) + kLeadElems;
+            tile2_f32<R, STAR, TY, TX>((const float*)P.src, (float*)P.dst, P.ny, P.nx, P.nx, P.bc, P.depth, cf, y0, x0, a,
+                                       a + TileGeom(R, P.depth, TY, TX).elems(), threadIdx.y * kBX + threadIdx.x, kBX * BY);
+        } else {
+            gather2d_tile<T, R, STAR, BY, TX, TY>((const T*)P.src, (T*)P.dst, P.ny, P.nx, P.nx, P.bc, P.depth, cf, y0, x0,
+                                                  reinterpret_cast<T*>(smem_raw));
+        }
     }
 }
 
@@ -305,21 +513,22 @@ __device__ __forceinline__ bool gwait(uint64_t* bar, uint32_t parity) {
     return ptx::mbar_wait(bar, parity, kGatherWait);
 }
 
-// 2D tile: TY x TX outputs per tile, threads (32, kBYT), NST stages in the
-// TMA ring (NST - 1 tiles in flight ahead of the one being computed).
-// FP32: 32 x 128, the last sub-step register-blocked (each thread kVR rows x
-// 4 columns: 256 threads cover the tile once), four stages (about 96 KB, two
-// CTAs per SM: six tiles in flight per SM); FP64: 64 x 32, one strip of kRS
-// rows per thread row, two stages.
+// 2D tile: TY x TX outputs per tile, threads (32, kBYT), a ring of TMA stages
+// (one less in flight ahead of the tile being computed).  FP32: 32 x 128
+// outputs (256 blocks of the last sub-step, one per thread); one step per
+// launch takes four stages (two CTAs of 96 KB per SM, six tiles in flight),
+// several steps two and a work buffer (72-78 KB: three CTAs per SM for depths
+// up to r tb = 4, so that one CTA's barriers and loads hide behind the
+// others' sub-steps).  FP64: 64 x 32, one strip of kRS rows per thread row,
+// two stages.
 template <typename T>
 struct Tile2 {
     static constexpr int TY = sizeof(T) == 4 ? 32 : 64;
     static constexpr int TX = sizeof(T) == 4 ? 128 : 32;
-    static constexpr int NST = sizeof(T) == 4 ? 4 : 2;
     static constexpr int AL = 16 / (int)sizeof(T);   // TMA x granule (16 bytes)
 };
-constexpr int kVR = 4;   // FP32 last sub-step: rows per thread
 constexpr int kBYT = 8;
+__host__ __device__ constexpr int stages2(size_t elem, bool multi) { return elem == 4 && !multi ? 4 : 2; }
 
 struct G2Args {
     const void* in;
@@ -330,9 +539,10 @@ struct G2Args {
     int tiles_x, tiles_total;
 };
 
-// Shared-memory layout of the 2D kernel for depth tb: NST stages (TMA ring)
-// and, for tb > 1, a work buffer for the sub-step ping-pong; kRS slack rows
-// after each buffer are read (never used) by ragged strips.
+// Shared-memory layout of the 2D kernel for depth tb: the TMA ring's stages
+// and, for tb > 1, a work buffer for the sub-step ping-pong; slack rows after
+// each buffer are read by ragged strips or blocks (FP32 blocks also write
+// them), never used.
 template <typename T>
 struct Layout2 {
     int H, HX, SY, SX, buf;   // halo rows, halo columns, rows, columns, elements per buffer
@@ -341,10 +551,11 @@ struct Layout2 {
         HX = round_up(H, Tile2<T>::AL);
         SY = Tile2<T>::TY + 2 * H;
         SX = Tile2<T>::TX + 2 * HX;
-        buf = round_up((SY + kRS) * SX, 128 / (int)sizeof(T));
+        buf = round_up((SY + (sizeof(T) == 4 ? kSlackRows : kRS)) * SX, 128 / (int)sizeof(T));
     }
-    __host__ __device__ int buffers(int tb) const { return Tile2<T>::NST + (tb > 1 ? 1 : 0); }
-    __host__ __device__ size_t bytes(int tb) const { return (size_t)buffers(tb) * buf * sizeof(T) + 64 + 128; }
+    __host__ __device__ int buffers(int tb) const { return stages2(sizeof(T), tb > 1) + (tb > 1 ? 1 : 0); }
+    // alignment slack, lead elements, buffers, barriers
+    __host__ __device__ size_t bytes(int tb) const { return 128 + 128 + (size_t)buffers(tb) * buf * sizeof(T) + 64; }
 };
 
 // One sub-step of depth t of the 2D tile: src -> dst (or -> the output grid
@@ -395,78 +606,6 @@ __device__ __forceinline__ void substep2(const T* src, T* dst, T* __restrict__ o
                         const bool outside = (bc == kBcDirichlet) && (gy < 0 || gy >= ny || gx < 0 || gx >= nx);
                         dst[sy * L.SX + sx] = outside ? T(0) : acc[j];
                     }
-                }
-            }
-        }
-    }
-}
-
-// Last sub-step of the 2D FP32 tile, register-blocked: a thread computes kRS
-// rows x 4 adjacent columns.  Each input row it needs is read as three 16-byte
-// shared-memory loads (columns x-4 .. x+7, enough for r <= 4), and every
-// weight is applied to four columns at once, so a update costs its P FMAs and
-// about one shared-memory load instruction (the scalar form spends about
-// 7.5 loads and the index arithmetic around them).  Rows of 4 outputs go out
-// as 16-byte stores.  The last sub-step's valid region starts at the aligned
-// column HX and is TX wide, so the column groups are aligned.
-template <int R, bool STAR>
-__device__ __forceinline__ void last_substep2_f32(const float* src, float* __restrict__ out, const Layout2<float>& L,
-                                                  int64_t ny, int64_t nx, int64_t ldx, int64_t y0, int64_t x0,
-                                                  const Coeffs<float, ipow(2 * R + 1, 2)>& cf) {
-    static_assert(R <= 4, "three 16-byte loads cover x-4 .. x+7");
-    constexpr int W = 2 * R + 1;
-    constexpr int kRS = kVR;   // rows per thread here
-    static_assert(Tile2<float>::TY % kRS == 0, "whole strips");
-    const int ncg = Tile2<float>::TX / 4;
-    const int nstrips = Tile2<float>::TY / kRS;
-    const int tid = threadIdx.y * kBX + threadIdx.x;
-    for (int item = tid; item < nstrips * ncg; item += kBX * kBYT) {
-        const int strip = item / ncg, cgi = item - strip * ncg;   // a warp: consecutive column groups
-        const int sy0 = L.H + strip * kRS;
-        const int sx = L.HX + 4 * cgi;
-        float acc[kRS][4];
-#pragma unroll
-        for (int j = 0; j < kRS; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
-        const float* base = src + (sy0 - R) * L.SX + (sx - 4);
-#pragma unroll
-        for (int yi = 0; yi < kRS + 2 * R; ++yi) {
-            float v[12];   // v[k] = column sx - 4 + k of input row sy0 - R + yi
-#pragma unroll
-            for (int k4 = 0; k4 < 3; ++k4) {
-                const float4 u = *reinterpret_cast<const float4*>(base + yi * L.SX + 4 * k4);
-                v[4 * k4] = u.x;
-                v[4 * k4 + 1] = u.y;
-                v[4 * k4 + 2] = u.z;
-                v[4 * k4 + 3] = u.w;
-            }
-#pragma unroll
-            for (int j = 0; j < kRS; ++j) {
-                const int a = yi - j;
-                if (a >= 0 && a < W) {
-#pragma unroll
-                    for (int b = 0; b < W; ++b)
-                        if (!STAR || a == R || b == R) {
-                            const float w = cf.c[a * W + b];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) acc[j][q] = fmaf(w, v[4 + q + b - R], acc[j][q]);
-                        }
-                }
-            }
-        }
-        const int64_t gx = x0 + 4 * cgi;
-#pragma unroll
-        for (int j = 0; j < kRS; ++j) {
-            const int64_t gy = y0 + strip * kRS + j;
-            if (gy < ny) {
-                float* o = out + gy * ldx + gx;
-                if (gx + 3 < nx) {
-                    *reinterpret_cast<float4*>(o) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (gx + q < nx) o[q] = acc[j][q];
                 }
             }
         }
@@ -543,18 +682,20 @@ __device__ __noinline__ void wrap_halo_block(T* buf, int SY, int SX, const T* __
 // the registers of one CTA, which at two spill some 600 bytes.)
 template <typename T, int NDIM>
 constexpr int min_ctas() { return sizeof(T) == 4 ? (NDIM == 2 ? 2 : 4) : 2; }
+template <typename T, int R, bool STAR, bool MULTI>
+constexpr int ctas2() { return sizeof(T) == 4 && MULTI ? (R == 1 ? 3 : R == 2 ? 2 : 1) : (STAR && R >= 4) ? 1 : min_ctas<T, 2>(); }
 
-template <typename T, int R, bool STAR>
-__global__ void __launch_bounds__(kBX * kBYT, (STAR && R >= 4) ? 1 : min_ctas<T, 2>())
+template <typename T, int R, bool STAR, bool MULTI>
+__global__ void __launch_bounds__(kBX * kBYT, (ctas2<T, R, STAR, MULTI>()))
 gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, const Coeffs<T, ipow(2 * R + 1, 2)> cf) {
     constexpr int TY = Tile2<T>::TY, TX = Tile2<T>::TX;
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char* smem_raw = (unsigned char*)(((uintptr_t)smem_dyn + 127) & ~(uintptr_t)127);
     const Layout2<T> L(R, a.tb);
-    constexpr int NST = Tile2<T>::NST;
-    T* const stage0 = reinterpret_cast<T*>(smem_raw);
+    constexpr int NST = stages2(sizeof(T), MULTI);
+    T* const stage0 = reinterpret_cast<T*>(smem_raw + kLeadElems * 4);
     T* work = stage0 + NST * L.buf;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + (size_t)L.buffers(a.tb) * L.buf * sizeof(T));
+    uint64_t* full = reinterpret_cast<uint64_t*>(stage0 + (size_t)L.buffers(a.tb) * L.buf);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(full + NST);
     const int tid = threadIdx.y * kBX + threadIdx.x;
     const T* in = (const T*)a.in;
@@ -611,19 +752,32 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
         }
         __syncthreads();
         if (*abort_flag) break;
-        T* src = st_buf;
-        for (int st = 1; st <= a.tb; ++st) {
-            T* dst = (st & 1) ? work : st_buf;   // sub-steps alternate between the work buffer and the stage
-            if constexpr (sizeof(T) == 4) {
-                if (st == a.tb)
-                    last_substep2_f32<R, STAR>(src, out, L, a.ny, a.nx, a.ldx, y0, x0, cf);
-                else
-                    substep2<T, R, STAR>(src, dst, out, L, st, false, a.ny, a.nx, a.ldx, a.bc, y0, x0, cf);
-            } else {
-                substep2<T, R, STAR>(src, dst, out, L, st, st == a.tb, a.ny, a.nx, a.ldx, a.bc, y0, x0, cf);
+        // sub-steps alternate between the work buffer and the stage
+        if constexpr (sizeof(T) == 4) {
+            const float* src = st_buf;
+            const TileGeom g(R, MULTI ? a.tb : 1, TY, TX);
+            if constexpr (MULTI) {
+                const int gy0 = (int)y0 - g.H, gx0 = (int)x0 - g.HX;
+                const bool zero = a.bc == kBcDirichlet &&
+                                  !(gy0 >= 0 && gy0 + g.SY <= a.ny && gx0 >= 0 && gx0 + g.SX <= a.nx);
+                for (int st = 1; st < a.tb; ++st) {
+                    float* dst = (st & 1) ? work : st_buf;
+                    substep_f32<R, STAR, TX>(src, dst, g, st, a.tb, zero, a.ny, a.nx, gy0, gx0, tid, kBX * kBYT, cf);
+                    src = dst;
+                    __syncthreads();
+                }
             }
-            src = dst;
-            __syncthreads();   // sub-step st is complete (and, after the last, the stage is free)
+            const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;   // rows are (TMA)
+            last_substep_f32<R, STAR, TY, TX>(src, out, g, vec, a.ny, a.nx, a.ldx, (int)y0, (int)x0, tid, kBX * kBYT, cf);
+            __syncthreads();   // the stage is free
+        } else {
+            T* src = st_buf;
+            for (int st = 1; st <= a.tb; ++st) {
+                T* dst = (st & 1) ? work : st_buf;
+                substep2<T, R, STAR>(src, dst, out, L, st, st == a.tb, a.ny, a.nx, a.ldx, a.bc, y0, x0, cf);
+                src = dst;
+                __syncthreads();   // sub-step st is complete (and, after the last, the stage is free)
+            }
         }
     }
     if (*abort_flag) {
@@ -809,7 +963,9 @@ constexpr int k3BY = 8, k3TX = 32, k3TY = 16, k3TZ = 8;
 constexpr int kBatchShapes = 2;
 constexpr int kBatchTY[kBatchShapes] = {64, 32};
 constexpr int kBatchTX[kBatchShapes] = {128, 64};
+constexpr int kBatchBY[kBatchShapes] = {8, 4};   // FP32: warps per CTA (two and one blocks per thread and sub-step)
 
+// What the deepest tile of a plan may take (a plan is refused beyond it).
 template <typename T>
 size_t gather_smem_bytes_t(int ndim, int r, int tb) {
     const int H = r * tb;
@@ -818,12 +974,21 @@ size_t gather_smem_bytes_t(int ndim, int r, int tb) {
     return (size_t)(nb * (k3TZ + 2 * H) + kRS) * (k3TY + 2 * H) * (k3TX + 2 * H) * sizeof(T);
 }
 
+// Shared memory of an element-loaded 2D tile (FP32: two blocked buffers; FP64:
+// the strips' layout).
+template <typename T>
+size_t tile2_smem_bytes(int r, int tb, int ty, int tx) {
+    if (sizeof(T) == 4) return (size_t)(kLeadElems + 2 * TileGeom(r, tb, ty, tx).elems()) * 4;
+    const int H = r * tb;
+    return (size_t)((tb > 1 ? 2 : 1) * (ty + 2 * H) + kRS) * (tx + 2 * H) * sizeof(T);
+}
+
 template <typename T, int R, bool STAR>
 cudaError_t launch2d_tiles(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
     constexpr int NC = ipow(2 * R + 1, 2);
     Coeffs<T, NC> cf;
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
-    const size_t smem = gather_smem_bytes_t<T>(2, R, tb);
+    const size_t smem = tile2_smem_bytes<T>(R, tb, k2TY, k2TX);
     auto kern = gather2d_kernel<T, R, STAR, k2BY, k2TX, k2TY>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -908,7 +1073,7 @@ cudaError_t launch2d(const GatherProblem& p, const void* in, void* out, int tb, 
     const cuuint64_t dims[2] = {(cuuint64_t)a.nx, (cuuint64_t)a.ny};
     const cuuint32_t box[2] = {(cuuint32_t)L.SX, (cuuint32_t)L.SY};
     if (!encode_grid_map<T>(&tin, in, 2, dims, p.ldx, box)) return cudaErrorInvalidValue;
-    auto kern = gather2d_tma_kernel<T, R, STAR>;
+    auto kern = tb > 1 ? gather2d_tma_kernel<T, R, STAR, true> : gather2d_tma_kernel<T, R, STAR, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per = 0;
@@ -984,28 +1149,27 @@ cudaError_t dispatch_r(const GatherProblem& p, const void* in, void* out, int tb
 
 template <typename T>
 size_t batch_smem_bytes_t(int r, int tb, int shape) {
-    const int H = r * tb;
-    const int nb = tb > 1 ? 2 : 1;
-    return (size_t)(nb * (kBatchTY[shape] + 2 * H) + kRS) * (kBatchTX[shape] + 2 * H) * sizeof(T);
+    return tile2_smem_bytes<T>(r, tb, kBatchTY[shape], kBatchTX[shape]);
 }
 
 template <typename T, int R, bool STAR, int S>
 cudaError_t launch_batch(const BatchProblem* probs, int nprob, int total_tiles, const void* coef, int max_tb,
                          int grid, cudaStream_t s) {
     const size_t smem = batch_smem_bytes_t<T>(R, max_tb, S);
-    auto kern = gather2d_batch_kernel<T, R, STAR, k2BY, kBatchTX[S], kBatchTY[S]>;
+    constexpr int BY = sizeof(T) == 4 ? kBatchBY[S] : k2BY;
+    auto kern = gather2d_batch_kernel<T, R, STAR, BY, kBatchTX[S], kBatchTY[S]>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (grid <= 0) {
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kBX * k2BY, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kBX * BY, smem);
         grid = sms * (per > 0 ? per : 1);
     }
     if (grid > total_tiles) grid = total_tiles;
     if (grid <= 0) return cudaSuccess;
-    kern<<<grid, dim3(kBX, k2BY), smem, s>>>(probs, nprob, total_tiles, (const T*)coef);
+    kern<<<grid, dim3(kBX, BY), smem, s>>>(probs, nprob, total_tiles, (const T*)coef);
     return cudaGetLastError();
 }
 
