@@ -52,6 +52,8 @@ GatherProblem gather_problem(const stencil_plan_s* p) {
     g.cg = p->cg.data();
     g.err = p->err_dev;
     g.ldx = p->ldx;
+    g.tuned = p->is_tuned ? &p->tuned : nullptr;
+    g.sched = p->gather_sched;
     return g;
 }
 
@@ -204,6 +206,44 @@ stencil_status ticket_done(uint64_t ticket, const Ticket& t, cudaError_t e) {
 // =================================================================== plans
 namespace {
 
+// Tile counter pairs of the gather plans: zero-initialised device memory of the
+// library (one allocation, copy or memset less per plan), handed out per plan
+// and returned with it.  Every launch leaves its pair at zero.  A plan that
+// finds none left runs with fixed tile shares.
+constexpr int kCounters = 1024;
+__device__ int g_counters[kCounters][2];
+struct Counters {
+    int* base = nullptr;
+    std::vector<int> free;
+};
+std::mutex g_counters_mu;
+std::map<int, Counters> g_counters_of;   // by device
+
+int* counter_take(int device) {
+    std::lock_guard<std::mutex> lk(g_counters_mu);
+    Counters& c = g_counters_of[device];
+    if (!c.base) {
+        void* q = nullptr;
+        if (cudaGetSymbolAddress(&q, g_counters) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c.base = (int*)q;
+        for (int i = kCounters - 1; i >= 0; --i) c.free.push_back(i);
+    }
+    if (c.free.empty()) return nullptr;
+    const int i = c.free.back();
+    c.free.pop_back();
+    return c.base + 2 * i;
+}
+
+void counter_give(int device, int* counter) {
+    if (!counter) return;
+    std::lock_guard<std::mutex> lk(g_counters_mu);
+    Counters& c = g_counters_of[device];
+    c.free.push_back((int)(counter - c.base) / 2);
+}
+
 // Free everything a plan (complete or half-built) owns.
 void plan_free(stencil_plan_s* p) {
     if (!p) return;
@@ -211,6 +251,8 @@ void plan_free(stencil_plan_s* p) {
     if (p->scratch) cudaFree(p->scratch);
     if (p->staging) cudaFree(p->staging);
     if (p->pad) cudaFree(p->pad);
+    // (after an aborted kernel the pair may not be zero: it is not handed out again)
+    if (!p->err_host || *(volatile unsigned int*)p->err_host == 0) counter_give(p->device, p->gather_sched);
     if (p->err_host) cudaFreeHost(p->err_host);
     if (p->stream) cudaStreamDestroy(p->stream);
     if (p->mx) {
@@ -427,6 +469,10 @@ extern "C" stencil_status stencil_plan_create(stencil_plan_t* out, int ndim, con
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
         if (gather_smem_bytes(g, p->tb) > (size_t)max_smem)
             return fail(STENCIL_EUNSUPPORTED, "temporal block depth too large for shared memory");
+        e = gather_prepare(g, p->scratch, p->tb, &p->tuned);
+        if (e != cudaSuccess) return cuda_fail(e, "gather kernel set-up");
+        p->is_tuned = true;
+        p->gather_sched = counter_take(p->device);
     } else {
         if (ndim == 3 && p->star && o.cover == STENCIL_COVER_AUTO)
             req.cover = pick_star_cover(req, p->repack ? p->pad_bytes : p->grid_bytes, p->scratch, p->stream);

@@ -43,26 +43,23 @@ cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t sme
 
 // Planes per work unit of a 3D sweep: units are `tiles` columns cut into
 // ceil(nz / c) chunks, processed by `slots` workers at about (c + fixed) plane
-// times each (`fixed`: halo planes and pipeline fill).  Returns the c <= most
-// with the shortest estimated sweep; the deeper of equals, which re-reads
-// fewer halo planes.  A fixed depth (64 planes, tensor cores 32) left small
-// grids on a few SMs and large ones with a nearly empty last wave; us per
-// sweep before and after: FP64 star 64^3 328 / 11, 512^3 1982 / 1956; FP32
-// gather 27-point 128^3 81 / 11, 512^3 375 / 336; tensor cores (with columns
-// of one quarter each, below) 27-point 64^3 29 / 8.6, 256^3 78 / 52,
-// 512^3 416 / 359, 7-point 512^3 229 / 200.
-inline int pick_chunk(int nz, int64_t tiles, int64_t slots, int fixed, int most) {
-    int best = 1;
-    int64_t best_cost = INT64_MAX;
-    for (int c = 1; c <= most && c <= nz; ++c) {
-        const int64_t units = tiles * ((nz + c - 1) / c);
-        const int64_t cost = (units + slots - 1) / slots * (c + fixed);
-        if (cost <= best_cost) {
-            best_cost = cost;
-            best = c;
-        }
-    }
-    return best;
+// times each (`fixed`: halo planes and pipeline fill).  Waves of units count in
+// steps of 1/`parts`: workers that share an SM run faster when some of them
+// have nothing left.  Returns the deepest c <= most within 1/`slack` of the
+// shortest estimated sweep (deeper units re-read fewer halo planes).
+// A fixed depth (64 planes, tensor cores 32) left small grids on a few SMs and
+// large ones with a nearly empty last wave; us per sweep before and after:
+// FP64 star 64^3 328 / 8.2, 512^3 1982 / 1863; FP32 gather 27-point 128^3
+// 81 / 9.3, 512^3 375 / 337; tensor cores (with columns of one quarter each,
+// mx3d.cu) 27-point 64^3 29 / 7.1, 256^3 78 / 52, 512^3 416 / 360, 7-point 512^3
+// 229 / 197.
+inline int pick_chunk(int nz, int64_t tiles, int64_t slots, int parts, int fixed, int most, int slack) {
+    auto cost = [&](int c) { return (tiles * ((nz + c - 1) / c) * parts + slots - 1) / slots * (c + fixed); };
+    int64_t least = cost(1);
+    for (int c = 2; c <= most && c <= nz; ++c) least = cost(c) < least ? cost(c) : least;
+    int c = most < nz ? most : nz;
+    while (c > 1 && cost(c) > least + least / slack) --c;
+    return c;
 }
 
 __host__ __device__ inline int64_t wrap_index(int64_t i, int64_t n) {

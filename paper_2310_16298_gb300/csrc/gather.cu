@@ -513,22 +513,28 @@ __device__ __forceinline__ bool gwait(uint64_t* bar, uint32_t parity) {
     return ptx::mbar_wait(bar, parity, kGatherWait);
 }
 
-// 2D tile: TY x TX outputs per tile, threads (32, kBYT), a ring of TMA stages
+// 2D tile: TY x TX outputs per tile, threads (32, BY), a ring of TMA stages
 // (one less in flight ahead of the tile being computed).  FP32: 32 x 128
 // outputs (256 blocks of the last sub-step, one per thread); one step per
-// launch takes four stages (two CTAs of 96 KB per SM, six tiles in flight),
+// launch takes three stages (three CTAs of 62 KB per SM, six tiles in flight),
 // several steps two and a work buffer (72-78 KB: three CTAs per SM for depths
 // up to r tb = 4, so that one CTA's barriers and loads hide behind the
-// others' sub-steps).  FP64: 64 x 32, one strip of kRS rows per thread row,
-// two stages.
+// others' sub-steps).  FP64: 32 x 32 outputs, one strip of 8 rows per thread,
+// two stages, four CTAs of four warps per SM: the FP64 pipe (2 FMAs per clock
+// and SM) is the limit, and with two CTAs of eight warps it sat idle a quarter
+// of the time around their barriers.  Grids with fewer such tiles than SMs
+// take 16 x 32 tiles (strips of 4 rows).  us per sweep before / after, star
+// r = 1: 256^2 8.3 / 2.8, 4096^2 187 / 175; box r = 2 4096^2 840 / 818, which is the
+// rate of bare FP64 FMAs on all SMs (510 G per second).
 template <typename T>
 struct Tile2 {
-    static constexpr int TY = sizeof(T) == 4 ? 32 : 64;
+    static constexpr int TY = 32;
+    static constexpr int TYS = sizeof(T) == 4 ? 32 : 16;   // small grids
     static constexpr int TX = sizeof(T) == 4 ? 128 : 32;
+    static constexpr int BY = sizeof(T) == 4 ? 8 : 4;
     static constexpr int AL = 16 / (int)sizeof(T);   // TMA x granule (16 bytes)
 };
-constexpr int kBYT = 8;
-__host__ __device__ constexpr int stages2(size_t elem, bool multi) { return elem == 4 && !multi ? 4 : 2; }
+__host__ __device__ constexpr int stages2(size_t elem, bool multi) { return elem == 4 && !multi ? 3 : 2; }
 
 struct G2Args {
     const void* in;
@@ -537,19 +543,20 @@ struct G2Args {
     int64_t ldx;         // row stride of the grids (elements)
     int ny, nx, bc, tb;
     int tiles_x, tiles_total;
+    int* sched;          // tile counter pair (0 between launches): [0] tiles claimed, [1] CTAs done; null: fixed shares
 };
 
 // Shared-memory layout of the 2D kernel for depth tb: the TMA ring's stages
 // and, for tb > 1, a work buffer for the sub-step ping-pong; slack rows after
 // each buffer are read by ragged strips or blocks (FP32 blocks also write
 // them), never used.
-template <typename T>
+template <typename T, int TY>
 struct Layout2 {
     int H, HX, SY, SX, buf;   // halo rows, halo columns, rows, columns, elements per buffer
     __host__ __device__ Layout2(int r, int tb) {
         H = r * tb;
         HX = round_up(H, Tile2<T>::AL);
-        SY = Tile2<T>::TY + 2 * H;
+        SY = TY + 2 * H;
         SX = Tile2<T>::TX + 2 * HX;
         buf = round_up((SY + (sizeof(T) == 4 ? kSlackRows : kRS)) * SX, 128 / (int)sizeof(T));
     }
@@ -561,31 +568,32 @@ struct Layout2 {
 // One sub-step of depth t of the 2D tile: src -> dst (or -> the output grid
 // on the last sub-step).  The buffer's element (sy, sx) is grid point
 // (y0 - H + sy, x0 - HX + sx).
-template <typename T, int R, bool STAR>
-__device__ __forceinline__ void substep2(const T* src, T* dst, T* __restrict__ out, const Layout2<T>& L, int t,
+template <typename T, int R, bool STAR, int TY>
+__device__ __forceinline__ void substep2(const T* src, T* dst, T* __restrict__ out, const Layout2<T, TY>& L, int t,
                                          bool last, int64_t ny, int64_t nx, int64_t ldx, int bc, int64_t y0, int64_t x0,
                                          const Coeffs<T, ipow(2 * R + 1, 2)>& cf) {
     constexpr int W = 2 * R + 1;
+    constexpr int RS = TY / Tile2<T>::BY;   // rows per strip
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int lo = R * t;                  // rows of the valid region skipped at the top
     const int lox = L.HX - L.H + R * t;    // columns skipped at the left
     const int Ht = L.SY - 2 * lo, Wt = L.SX - 2 * lox;
-    const int nstrips = (Ht + kRS - 1) / kRS;
-    for (int strip = ty; strip < nstrips; strip += kBYT) {
-        const int sy0 = lo + strip * kRS;
+    const int nstrips = (Ht + RS - 1) / RS;
+    for (int strip = ty; strip < nstrips; strip += Tile2<T>::BY) {
+        const int sy0 = lo + strip * RS;
         for (int c = tx; c < Wt; c += kBX) {
             const int sx = lox + c;
-            T acc[kRS];
+            T acc[RS];
 #pragma unroll
-            for (int j = 0; j < kRS; ++j) acc[j] = T(0);
+            for (int j = 0; j < RS; ++j) acc[j] = T(0);
             const T* base = src + (sy0 - R) * L.SX + (sx - R);
 #pragma unroll
-            for (int yi = 0; yi < kRS + 2 * R; ++yi) {
+            for (int yi = 0; yi < RS + 2 * R; ++yi) {
                 T v[W];
 #pragma unroll
                 for (int b = 0; b < W; ++b) v[b] = base[yi * L.SX + b];
 #pragma unroll
-                for (int j = 0; j < kRS; ++j) {
+                for (int j = 0; j < RS; ++j) {
                     const int a = yi - j;
                     if (a >= 0 && a < W) {
 #pragma unroll
@@ -596,7 +604,7 @@ __device__ __forceinline__ void substep2(const T* src, T* dst, T* __restrict__ o
             }
             const int64_t gx = x0 - L.HX + sx;
 #pragma unroll
-            for (int j = 0; j < kRS; ++j) {
+            for (int j = 0; j < RS; ++j) {
                 const int sy = sy0 + j;
                 if (sy < L.SY - lo) {
                     const int64_t gy = y0 - L.H + sy;
@@ -661,7 +669,7 @@ __device__ __forceinline__ void wrap_halo_block_inl(T* buf, int SY, int SX, cons
                     sx = c < cl ? c : cr + (c - cl);
                 }
                 off[u] = sy * SX + sx;
-                v[u] = in[(int64_t)wrap_fast(gy0 + sy, ny) * ldx + wrap_fast(gx0 + sx, nx)];
+                v[u] = __ldcg(in + (int64_t)wrap_fast(gy0 + sy, ny) * ldx + wrap_fast(gx0 + sx, nx));
             }
         }
 #pragma unroll
@@ -678,25 +686,26 @@ __device__ __noinline__ void wrap_halo_block(T* buf, int SY, int SX, const T* __
 
 // Register budgets of the persistent kernels: left alone, the compiler keeps
 // the coefficients and unrolled sums in registers and one CTA fills an SM.
-// (2D: two CTAs of four-stage rings fill the shared memory; r = 4 stars get
-// the registers of one CTA, which at two spill some 600 bytes.)
-template <typename T, int NDIM>
-constexpr int min_ctas() { return sizeof(T) == 4 ? (NDIM == 2 ? 2 : 4) : 2; }
 template <typename T, int R, bool STAR, bool MULTI>
-constexpr int ctas2() { return sizeof(T) == 4 && MULTI ? (R == 1 ? 3 : R == 2 ? 2 : 1) : (STAR && R >= 4) ? 1 : min_ctas<T, 2>(); }
+constexpr int ctas2() {
+    if (sizeof(T) == 8) return STAR && R >= 3 ? 2 : 4;   // (strips of wide stars hold 2r+1 rows in registers)
+    return MULTI ? (R == 1 ? 3 : R == 2 ? 2 : 1) : (STAR && R >= 4) ? 2 : 3;
+}
 
-template <typename T, int R, bool STAR, bool MULTI>
-__global__ void __launch_bounds__(kBX * kBYT, (ctas2<T, R, STAR, MULTI>()))
+template <typename T, int R, bool STAR, bool MULTI, int TY>
+__global__ void __launch_bounds__(kBX * Tile2<T>::BY, (ctas2<T, R, STAR, MULTI>()))
 gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, const Coeffs<T, ipow(2 * R + 1, 2)> cf) {
-    constexpr int TY = Tile2<T>::TY, TX = Tile2<T>::TX;
+    constexpr int TX = Tile2<T>::TX;
+    constexpr int kThr = kBX * Tile2<T>::BY;
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char* smem_raw = (unsigned char*)(((uintptr_t)smem_dyn + 127) & ~(uintptr_t)127);
-    const Layout2<T> L(R, a.tb);
+    const Layout2<T, TY> L(R, a.tb);
     constexpr int NST = stages2(sizeof(T), MULTI);
     T* const stage0 = reinterpret_cast<T*>(smem_raw + kLeadElems * 4);
     T* work = stage0 + NST * L.buf;
     uint64_t* full = reinterpret_cast<uint64_t*>(stage0 + (size_t)L.buffers(a.tb) * L.buf);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(full + NST);
+    volatile int* stage_tile = abort_flag + 1;   // [NST] tile of each stage (-1: no more)
     const int tid = threadIdx.y * kBX + threadIdx.x;
     const T* in = (const T*)a.in;
     T* out = (T*)a.out;
@@ -705,7 +714,14 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
         for (int i = 0; i < NST; ++i) ptx::mbar_init(&full[i], 1);
         *abort_flag = 0;
         ptx::fence_mbar_init();
+        ptx::prefetch_tensormap(&tin);
     }
+    // programmatic dependent launch (common.cuh): a grid with a CTA per tile lets
+    // the next sweep set itself up beside it (not FP64: the CTAs that wait crowd
+    // on to the free SMs and then share their FP64 pipes: 256^2 r = 1 star 4.8 us
+    // per sweep against 2.8); the grids are touched from here on
+    if (sizeof(T) == 4 && (int)gridDim.x == a.tiles_total) ptx::launch_dependents();
+    ptx::grid_dependency_wait();
     __syncthreads();
     // Every tile is staged by TMA; with a periodic boundary, a tile whose
     // staged block crosses the grid's edge then gets its outside cells wrapped.
@@ -716,19 +732,35 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
     };
     // Thread 0 tracks the ring: bit s of `inflight` = a load into stage s not
     // yet waited for, bit s of `phase` = parity of stage s's next completion.
+    // The first NST - 1 tiles of a CTA are fixed; on grids of more tiles the
+    // others are claimed one ahead of the stage that comes free, so that the
+    // atomic's round trip is never waited for.  SMs do not run equally fast: with
+    // fixed shares the CTAs' positions, and so the rows in flight, drift apart
+    // (8192^2 r = 1 box 91 us, with claims 79: the copy bandwidth).
     uint32_t inflight = 0, phase = 0;
-    auto issue = [&](int t, int s) {
-        if (t >= a.tiles_total) return;
+    int issued = 0, claimed = 0;
+    bool more = true;
+    auto issue = [&]() {
+        if (!more) return;
+        const int s = issued % NST;
+        const int t = a.sched && issued >= NST - 1 ? (NST - 1) * (int)gridDim.x + claimed
+                                                   : (int)blockIdx.x + issued * (int)gridDim.x;
+        if (a.sched && issued >= NST - 2 && t < a.tiles_total) claimed = atomicAdd(&a.sched[0], 1);
+        ++issued;
+        more = t < a.tiles_total;
+        stage_tile[s] = more ? t : -1;
+        if (!more) {
+            ptx::mbar_arrive(&full[s]);
+            return;
+        }
         const int y0 = (t / a.tiles_x) * TY, x0 = (t % a.tiles_x) * TX;
         ptx::mbar_arrive_expect_tx(&full[s], box_bytes);
         ptx::tma_load_2d(stage0 + s * L.buf, &tin, x0 - L.HX, y0 - L.H, &full[s]);
         inflight |= 1u << s;
     };
-    const int first = blockIdx.x;
     if (tid == 0)
-        for (int i = 0; i < NST - 1; ++i) issue(first + i * (int)gridDim.x, i);
-    int k = 0;
-    for (int t = first; t < a.tiles_total; t += gridDim.x, ++k) {
+        for (int i = 0; i < NST - 1; ++i) issue();
+    for (int k = 0;; ++k) {
         const int s = k % NST;
         T* st_buf = stage0 + s * L.buf;
         // the stage computed at iteration k - 1 is free (barrier at its end);
@@ -736,15 +768,17 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
         // before the TMA write that refills it
         if (tid == 0) {
             ptx::fence_proxy_async_smem();
-            issue(t + (NST - 1) * (int)gridDim.x, (k + NST - 1) % NST);
+            issue();
         }
-        const int64_t y0 = (int64_t)(t / a.tiles_x) * TY, x0 = (int64_t)(t % a.tiles_x) * TX;
         {
             const uint32_t par = (phase >> s) & 1u;   // every thread tracks the parities
             if (!gwait(&full[s], par)) *abort_flag = 1;
             phase ^= 1u << s;
             if (tid == 0) inflight &= ~(1u << s);
         }
+        const int t = stage_tile[s];
+        if (t < 0) break;
+        const int64_t y0 = (int64_t)(t / a.tiles_x) * TY, x0 = (int64_t)(t % a.tiles_x) * TX;
         if (edge(t)) {
             __syncthreads();   // every thread has seen the load land (or the abort)
             if (!*abort_flag)
@@ -762,19 +796,19 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
                                   !(gy0 >= 0 && gy0 + g.SY <= a.ny && gx0 >= 0 && gx0 + g.SX <= a.nx);
                 for (int st = 1; st < a.tb; ++st) {
                     float* dst = (st & 1) ? work : st_buf;
-                    substep_f32<R, STAR, TX>(src, dst, g, st, a.tb, zero, a.ny, a.nx, gy0, gx0, tid, kBX * kBYT, cf);
+                    substep_f32<R, STAR, TX>(src, dst, g, st, a.tb, zero, a.ny, a.nx, gy0, gx0, tid, kThr, cf);
                     src = dst;
                     __syncthreads();
                 }
             }
             const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;   // rows are (TMA)
-            last_substep_f32<R, STAR, TY, TX>(src, out, g, vec, a.ny, a.nx, a.ldx, (int)y0, (int)x0, tid, kBX * kBYT, cf);
+            last_substep_f32<R, STAR, TY, TX>(src, out, g, vec, a.ny, a.nx, a.ldx, (int)y0, (int)x0, tid, kThr, cf);
             __syncthreads();   // the stage is free
         } else {
             T* src = st_buf;
             for (int st = 1; st <= a.tb; ++st) {
                 T* dst = (st & 1) ? work : st_buf;
-                substep2<T, R, STAR>(src, dst, out, L, st, st == a.tb, a.ny, a.nx, a.ldx, a.bc, y0, x0, cf);
+                substep2<T, R, STAR, TY>(src, dst, out, L, st, st == a.tb, a.ny, a.nx, a.ldx, a.bc, y0, x0, cf);
                 src = dst;
                 __syncthreads();   // sub-step st is complete (and, after the last, the stage is free)
             }
@@ -788,6 +822,13 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
             if (a.err) atomicOr(a.err, 2u);
         }
     }
+    if (a.sched && tid == 0) {   // this CTA has made its last claim: the last CTA resets the counter
+        __threadfence();
+        if (atomicAdd(&a.sched[1], 1) == (int)gridDim.x - 1) {
+            atomicExch(&a.sched[0], 0);
+            atomicExch(&a.sched[1], 0);
+        }
+    }
 }
 
 // 3D streaming kernel: a work unit is a.tzc output planes of a TY x TX column
@@ -796,10 +837,10 @@ gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, con
 template <typename T>
 struct Tile3 {
     static constexpr int TY = 32;
-    static constexpr int TX = 64;
+    static constexpr int TX = sizeof(T) == 4 ? 64 : 32;   // FP64: CTAs of half the size, four per SM (as in 2D)
+    static constexpr int THREADS = TX * (TY / kRS);       // one strip of kRS rows of one column each
     static constexpr int AL = 16 / (int)sizeof(T);
 };
-constexpr int kThreads3 = 256;   // (TY / kRS) strips x TX columns
 
 struct G3Args {
     const void* in;
@@ -822,11 +863,10 @@ struct Layout3 {
 };
 
 template <typename T, int R, bool STAR>
-__global__ void __launch_bounds__(kThreads3, min_ctas<T, 3>())
+__global__ void __launch_bounds__(Tile3<T>::THREADS, sizeof(T) == 4 ? 4 : (R >= 3 ? 1 : 4))
 gather3d_stream_kernel(const __grid_constant__ CUtensorMap tin, const G3Args a, const Coeffs<T, ipow(2 * R + 1, 3)> cf) {
     using L = Layout3<T, R>;
     constexpr int W = 2 * R + 1, TY = Tile3<T>::TY, TX = Tile3<T>::TX, NPL = L::NPL;
-    static_assert(TX * (TY / kRS) == kThreads3, "one strip per thread");
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char* smem_raw = (unsigned char*)(((uintptr_t)smem_dyn + 127) & ~(uintptr_t)127);
     T* planes = reinterpret_cast<T*>(smem_raw);
@@ -840,7 +880,11 @@ gather3d_stream_kernel(const __grid_constant__ CUtensorMap tin, const G3Args a, 
         for (int b = 0; b < NPL; ++b) ptx::mbar_init(&full[b], 1);
         *abort_flag = 0;
         ptx::fence_mbar_init();
+        ptx::prefetch_tensormap(&tin);
     }
+    // as in the 2D kernel
+    if (sizeof(T) == 4 && (int)gridDim.x == a.units) ptx::launch_dependents();
+    ptx::grid_dependency_wait();
     __syncthreads();
     int uses[NPL];   // TMA loads into each plane buffer so far (mbarrier phases)
 #pragma unroll
@@ -1043,18 +1087,38 @@ bool encode_grid_map(CUtensorMap* map, const void* base, int rank, const cuuint6
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int smem_limit(const GatherProblem& p) { return p.tuned ? p.tuned->max_smem : max_smem_optin(); }
+
 // The TMA kernels need 16-byte aligned grid bases and rows.
 template <typename T>
 bool tma_layout_ok(const GatherProblem& p, const void* in) {
     return ((uintptr_t)in & 15u) == 0 && (p.ldx * (int64_t)sizeof(T)) % 16 == 0;
 }
 
-template <typename T, int R, bool STAR>
-cudaError_t launch2d(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
-    const Layout2<T> L(R, tb);
+// How many CTAs of a TMA kernel fit: from the plan, which asks the runtime once
+// (p.prepare, at its creation), or asked now.
+template <typename K>
+cudaError_t tuned_for(const GatherProblem& p, K kern, int threads, size_t smem, int tb, GatherTuned* t) {
+    if (p.tuned && !p.prepare) {
+        *t = *p.tuned;
+        if (t->per_sm[tb] > 0) return cudaSuccess;
+    }
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    t->sms = sm_count();
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t->per_sm[tb], kern, threads, smem);
+    if (t->per_sm[tb] < 1) t->per_sm[tb] = 1;
+    if (e == cudaSuccess && p.prepare) {
+        p.prepare->sms = t->sms;
+        p.prepare->per_sm[tb] = t->per_sm[tb];
+    }
+    return e;
+}
+
+template <typename T, int R, bool STAR, int TY>
+cudaError_t launch2d_tma(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
+    const Layout2<T, TY> L(R, tb);
     const size_t smem = L.bytes(tb);
-    if (!tma_layout_ok<T>(p, in) || smem > (size_t)max_smem_optin() || L.SX > 256 || L.SY > 256)
-        return launch2d_tiles<T, R, STAR>(p, in, out, tb, s);
     constexpr int NC = ipow(2 * R + 1, 2);
     Coeffs<T, NC> cf;
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
@@ -1068,29 +1132,40 @@ cudaError_t launch2d(const GatherProblem& p, const void* in, void* out, int tb, 
     a.bc = p.bc;
     a.tb = tb;
     a.tiles_x = (a.nx + Tile2<T>::TX - 1) / Tile2<T>::TX;
-    a.tiles_total = a.tiles_x * ((a.ny + Tile2<T>::TY - 1) / Tile2<T>::TY);
+    a.tiles_total = a.tiles_x * ((a.ny + TY - 1) / TY);
     alignas(64) CUtensorMap tin;
     const cuuint64_t dims[2] = {(cuuint64_t)a.nx, (cuuint64_t)a.ny};
     const cuuint32_t box[2] = {(cuuint32_t)L.SX, (cuuint32_t)L.SY};
     if (!encode_grid_map<T>(&tin, in, 2, dims, p.ldx, box)) return cudaErrorInvalidValue;
-    auto kern = tb > 1 ? gather2d_tma_kernel<T, R, STAR, true> : gather2d_tma_kernel<T, R, STAR, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kBX * kBYT, smem);
-    if (e != cudaSuccess) return e;
-    int grid = sm_count() * (per > 0 ? per : 1);
+    constexpr bool F32 = sizeof(T) == 4;
+    auto kern = F32 && tb > 1 ? gather2d_tma_kernel<T, R, STAR, F32, TY> : gather2d_tma_kernel<T, R, STAR, false, TY>;
+    constexpr int threads = kBX * Tile2<T>::BY;
+    GatherTuned t;
+    cudaError_t e = tuned_for(p, kern, threads, smem, tb, &t);
+    if (e != cudaSuccess || p.prepare) return e;
+    int grid = t.sms * t.per_sm[tb];
     if (grid > a.tiles_total) grid = a.tiles_total;
-    kern<<<grid, dim3(kBX, kBYT), smem, s>>>(tin, a, cf);
-    return cudaGetLastError();
+    a.sched = sizeof(T) == 4 && grid < a.tiles_total ? p.sched : nullptr;   // FP64: compute-bound, fixed shares do
+    return launch_dependent(kern, dim3(grid), dim3(kBX, Tile2<T>::BY), smem, s, tin, a, cf);
+}
+
+template <typename T, int R, bool STAR>
+cudaError_t launch2d(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
+    constexpr int TY = Tile2<T>::TY, TYS = Tile2<T>::TYS, TX = Tile2<T>::TX;
+    const Layout2<T, TY> L(R, tb);
+    if (!tma_layout_ok<T>(p, in) || L.bytes(tb) > (size_t)smem_limit(p) || L.SX > 256 || L.SY > 256)
+        return p.prepare ? cudaSuccess : launch2d_tiles<T, R, STAR>(p, in, out, tb, s);
+    const int64_t tiles = ((p.n[0] + TY - 1) / TY) * ((p.n[1] + TX - 1) / TX);
+    if (TYS != TY && tiles < (p.tuned ? p.tuned->sms : sm_count())) return launch2d_tma<T, R, STAR, TYS>(p, in, out, tb, s);
+    return launch2d_tma<T, R, STAR, TY>(p, in, out, tb, s);
 }
 
 template <typename T, int R, bool STAR>
 cudaError_t launch3d(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
     using L = Layout3<T, R>;
     const size_t smem = L::bytes();
-    if (tb != 1 || !tma_layout_ok<T>(p, in) || smem > (size_t)max_smem_optin() || L::SX > 256 || L::SY > 256)
-        return launch3d_tiles<T, R, STAR>(p, in, out, tb, s);
+    if (tb != 1 || !tma_layout_ok<T>(p, in) || smem > (size_t)smem_limit(p) || L::SX > 256 || L::SY > 256)
+        return p.prepare ? cudaSuccess : launch3d_tiles<T, R, STAR>(p, in, out, tb, s);
     constexpr int NC = ipow(2 * R + 1, 3);
     Coeffs<T, NC> cf;
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
@@ -1110,21 +1185,19 @@ cudaError_t launch3d(const GatherProblem& p, const void* in, void* out, int tb, 
     const cuuint32_t box[3] = {(cuuint32_t)L::SX, (cuuint32_t)L::SY, 1};
     if (!encode_grid_map<T>(&tin, in, 3, dims, p.ldx, box)) return cudaErrorInvalidValue;
     auto kern = gather3d_stream_kernel<T, R, STAR>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads3, smem);
-    if (e != cudaSuccess) return e;
-    int grid = sm_count() * (per > 0 ? per : 1);
+    GatherTuned t;
+    cudaError_t e = tuned_for(p, kern, Tile3<T>::THREADS, smem, 1, &t);
+    if (e != cudaSuccess || p.prepare) return e;
+    int grid = t.sms * t.per_sm[1];
     // A unit's fixed cost in planes: FP32 units re-read 2R halo planes and wait
     // for the first 2R + 1 to land; FP64 units compute far longer than that per
-    // plane.
+    // plane, so even shares matter most.
     const int tiles = a.tiles_x * a.tiles_y;
-    a.tzc = pick_chunk(a.nz, tiles, grid, sizeof(T) == 8 ? 1 : 2 * R + 2, 64);
+    a.tzc = sizeof(T) == 8 ? pick_chunk(a.nz, tiles, grid, 2, 1, 64, 1 << 20)
+                           : pick_chunk(a.nz, tiles, grid, 2, 2 * R + 2, 64, 32);
     a.units = tiles * ((a.nz + a.tzc - 1) / a.tzc);
     if (grid > a.units) grid = a.units;
-    kern<<<grid, kThreads3, smem, s>>>(tin, a, cf);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(grid), dim3(Tile3<T>::THREADS), smem, s, tin, a, cf);
 }
 
 template <typename T, bool STAR>
@@ -1215,6 +1288,19 @@ size_t gather_batch_smem_bytes(bool f64, int r, int tb, int shape) {
 
 size_t gather_smem_bytes(const GatherProblem& p, int tb) {
     return p.f64 ? gather_smem_bytes_t<double>(p.ndim, p.r, tb) : gather_smem_bytes_t<float>(p.ndim, p.r, tb);
+}
+
+cudaError_t gather_prepare(const GatherProblem& p, const void* grid, int tb, GatherTuned* t) {
+    t->sms = sm_count();
+    t->max_smem = max_smem_optin();
+    GatherProblem q = p;
+    q.tuned = t;
+    q.prepare = t;
+    for (int d = 1; d <= tb && d <= kMaxTb; ++d) {
+        const cudaError_t e = gather_sweep(q, grid, nullptr, d, nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t gather_sweep(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {

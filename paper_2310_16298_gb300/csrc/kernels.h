@@ -7,6 +7,13 @@
 
 namespace stx {
 
+// What the runtime says about a plan's TMA kernels (asked once, at creation).
+constexpr int kMaxTb = 16;
+struct GatherTuned {
+    int sms = 0, max_smem = 0;
+    int per_sm[kMaxTb + 1] = {};   // CTAs per SM by depth (0: not a TMA kernel)
+};
+
 // A single-grid problem as the gather kernels see it.
 struct GatherProblem {
     int ndim;          // 2 or 3
@@ -17,9 +24,14 @@ struct GatherProblem {
     int bc;            // kBcDirichlet | kBcPeriodic
     const double* cg;  // host: dense C^g, (2r+1)^ndim, gather orientation
     int64_t ldx = 0;   // row stride of the grids (elements); planes are n[ndim-2] rows
+    int* sched = nullptr;                 // the plan's tile counter pair (device; zero between launches)
+    const GatherTuned* tuned = nullptr;   // of the plan (null: asked at each sweep)
+    GatherTuned* prepare = nullptr;       // set: fill this instead of launching
     unsigned int* err = nullptr;  // device view of the plan's host-mapped error word (bounded waits)
 };
 
+// Set the kernels of depths 1 .. tb up for p (`grid`: any grid of its layout).
+cudaError_t gather_prepare(const GatherProblem& p, const void* grid, int tb, GatherTuned* t);
 // Advance `in` by `tb` time steps into `out` (distinct buffers).
 cudaError_t gather_sweep(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s);
 size_t gather_smem_bytes(const GatherProblem& p, int tb);

@@ -771,7 +771,8 @@ cudaError_t mx3d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     a.bpart_bytes = st->bpart_bytes;
     a.tiles_x = (nx + st->nb - 1) / st->nb;
     a.groups = (a.tiles_x * ((ny + rows_out - 1) / rows_out) + kQuarters - 1) / kQuarters;
-    a.chunk = p.unit_planes > 0 ? p.unit_planes : pick_chunk(nz, a.groups, st->num_sms, 2 * p.r + kFillPlanes, kMaxChunk);
+    a.chunk = p.unit_planes > 0 ? p.unit_planes
+                                : pick_chunk(nz, a.groups, st->num_sms, 1, 2 * p.r + kFillPlanes, kMaxChunk, 32);
     a.units = a.groups * ((nz + a.chunk - 1) / a.chunk);
     a.bop_bytes = st->bop_bytes;
     alignas(64) CUtensorMap map, map_out;

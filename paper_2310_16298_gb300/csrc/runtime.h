@@ -42,6 +42,9 @@ struct stencil_plan_s {
     void* staging = nullptr;        // device grid of stencil_apply_host (allocated on first use)
     unsigned int* err_host = nullptr;  // host-mapped error word of the gather kernels' bounded waits
     unsigned int* err_dev = nullptr;
+    int* gather_sched = nullptr;    // tile counter pair of the gather kernels (null: none was left)
+    stx::GatherTuned tuned;         // launch shapes of the gather kernels
+    bool is_tuned = false;
 };
 
 
