@@ -65,7 +65,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <array>
 #include <cmath>
 #include <type_traits>
 #include <vector>
@@ -116,6 +115,17 @@ struct Pair {
     static constexpr int NBLK = 2 * NBP;
     // lane offset d of block (p, i) is dlo(p) + i
     __host__ __device__ static constexpr int dlo(int p) { return -((R + 1 - p) / 2); }
+    // Place of block (p, i) along N.  Two blocks hold one line only (a line past
+    // either end stands where their other one would): (e, R) uses even input
+    // rows only, (1 - e, 0) odd rows only, e = R mod 2.  The first comes first
+    // and the second last, so that each row parity's MMAs run on the NBLK - 1
+    // adjacent blocks that use it (issue_pair_products).
+    __host__ __device__ static constexpr int pos(int p, int i) {
+        return p == R % 2 && i == R          ? 0
+               : p != R % 2 && i == 0        ? NBLK - 1
+               : R % 2 == 0 ? (p == 0 ? 1 + i : R + i)
+                            : (p == 0 ? i : R + 1 + i);
+    }
 };
 
 template <bool BF>
@@ -293,6 +303,57 @@ __device__ __forceinline__ void boundary_strips(const MxArgs2D& a, int first, in
     }
 }
 
+// The products of one item (as issue_products), each row parity's K steps on
+// the blocks that use it: N - 16 of the N columns, the even rows' from block 0
+// and the odd rows' from block 1 (the first MMA runs on all, to clear them).
+// The columns left out would add zeros.  8192^2 TF32x3, us per sweep with all
+// columns / without: order 4 128 / 124, order 3 112 / 110.
+template <bool BF, int KS, int N, int PA, int PB, bool FIRST>
+__device__ __forceinline__ void issue_pair_product(uint32_t d, uint32_t a_base, int part_cols, uint64_t b_desc0,
+                                                   uint32_t bpart_bytes) {
+    constexpr uint32_t F = OpFmt<BF>::kFmt;
+    constexpr uint32_t all = ptx::instr_desc(F, F, 128, (uint32_t)N);
+    constexpr uint32_t most = ptx::instr_desc(F, F, 128, (uint32_t)(N - kNb));
+    const uint32_t a = a_base + (uint32_t)(PA * part_cols);
+    const uint64_t b = b_desc0 + (uint64_t)((PB * bpart_bytes) >> 4);
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+        const uint64_t bd = b + (uint64_t)((2 * ks * N * 16) >> 4);
+        if (FIRST && ks == 0)
+            ptx::mma_ts<BF, true>(d, a + 8 * ks, bd, all);
+        else if (ks < KS / 2)
+            ptx::mma_ts<BF, false>(d, a + 8 * ks, bd, most);
+        else
+            ptx::mma_ts<BF, false>(d + kNb, a + 8 * ks, bd + kNb, most);   // 16 rows of 16 bytes on
+    }
+}
+
+template <bool BF, int KS, int N>
+__device__ __forceinline__ void issue_pair_products(uint32_t d, uint32_t a, int pc, uint64_t b0, uint32_t bpb, int nprod) {
+    switch (nprod) {
+        case 1:
+            issue_pair_product<BF, KS, N, 0, 0, true>(d, a, pc, b0, bpb);
+            break;
+        case 2:
+            issue_pair_product<BF, KS, N, 0, 1, true>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 0, 0, false>(d, a, pc, b0, bpb);
+            break;
+        case 3:
+            issue_pair_product<BF, KS, N, 1, 0, true>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 0, 1, false>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 0, 0, false>(d, a, pc, b0, bpb);
+            break;
+        case 6:
+            issue_pair_product<BF, KS, N, 0, 2, true>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 1, 1, false>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 2, 0, false>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 1, 0, false>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 0, 1, false>(d, a, pc, b0, bpb);
+            issue_pair_product<BF, KS, N, 0, 0, false>(d, a, pc, b0, bpb);
+            break;
+    }
+}
+
 template <int R, bool BF, int NP>
 __global__ void __launch_bounds__(kThreads, 1)
 mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ CUtensorMap tmap_o,
@@ -438,7 +499,6 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
         // ------------------------------------------------ MMA issuers (items i with i % 2 == u)
         const int u = warp == 1 ? 0 : 1;
         if (lane == 0 && wait_or_abort(bop_bar, 0, abort_flag)) {
-            constexpr uint32_t idesc = ptx::instr_desc(F::kFmt, F::kFmt, 128, (uint32_t)N);
             const uint64_t b0 = ptx::smem_desc(ptx::smem_u32(bops), (uint32_t)(N * 16), 128);
             const int pr = args.nprod;
             for (int i = u;; i += 2) {
@@ -450,8 +510,8 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                 if (a_tile[sa] < 0) break;   // the split warps passed the end of the tiles
                 if (!wait_or_abort(&acce[st], ph ^ 1u, abort_flag)) break;
                 ptx::tc_fence_after();
-                issue_products<BF, KS>(tmem_d + (uint32_t)(st * N), tmem_a + (uint32_t)(sa * A_COLS), PC, b0,
-                                       args.bpart_bytes, N, idesc, pr);
+                issue_pair_products<BF, KS, N>(tmem_d + (uint32_t)(st * N), tmem_a + (uint32_t)(sa * A_COLS), PC, b0,
+                                               args.bpart_bytes, pr);
                 ptx::mma_commit(&aempty[sa]);
                 ptx::mma_commit(&accf[st]);
                 committed = i;
@@ -558,7 +618,8 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                 ptx::tc_fence_after();
                 const int X0 = (t % args.tiles_x) * kTw;   // in the tiles' region
                 const int Y0 = (t / args.tiles_x) * (kQuarters * G::ROWS_OUT);
-                const uint32_t dbase = tmem_d + lane_off + (uint32_t)(st * N + P * G::NBP * kNb);
+                const uint32_t dbase = tmem_d + lane_off + (uint32_t)(st * N);
+                auto block = [&](int i) { return dbase + (uint32_t)(G::pos(P, i) * kNb); };
                 float acc[kNb];
 #pragma unroll
                 for (int b0 = 0; b0 < G::NBP; b0 += LB) {
@@ -568,17 +629,15 @@ mx2d_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ 
                     uint32_t v[LB][kNb];
                     uint32_t v0[kNb];
                     const int nv = G::NBP - b0 < LB ? G::NBP - b0 : LB;
-                    const uint32_t ba = dbase + (uint32_t)(b0 * kNb);
-                    const uint32_t bi = dbase + (uint32_t)(I0 * kNb);
                     if (b0 == 0 && I0 >= LB) {
-                        if (nv == 2) ptx::tmem_ld_x16_sync(ba, v[0], ba + kNb, v[1], bi, v0);
-                        if (nv == 1) ptx::tmem_ld_x16_sync(ba, v[0], bi, v0);
+                        if (nv == 2) ptx::tmem_ld_x16_sync(block(0), v[0], block(1), v[1], block(I0), v0);
+                        if (nv == 1) ptx::tmem_ld_x16_sync(block(0), v[0], block(I0), v0);
                     } else {
                         if constexpr (LB >= 3) {
-                            if (nv == 3) ptx::tmem_ld_x16_sync(ba, v[0], ba + kNb, v[1], ba + 2 * kNb, v[2]);
+                            if (nv == 3) ptx::tmem_ld_x16_sync(block(b0), v[0], block(b0 + 1), v[1], block(b0 + 2), v[2]);
                         }
-                        if (nv == 2) ptx::tmem_ld_x16_sync(ba, v[0], ba + kNb, v[1]);
-                        if (nv == 1) ptx::tmem_ld_x16_sync(ba, v[0]);
+                        if (nv == 2) ptx::tmem_ld_x16_sync(block(b0), v[0], block(b0 + 1), v[1]);
+                        if (nv == 1) ptx::tmem_ld_x16_sync(block(b0), v[0]);
                     }
                     if (b0 + LB >= G::NBP) {   // last batch: the accumulator set is free
                         ptx::tc_fence_before();
@@ -704,23 +763,32 @@ KernelInfo kernel_for(int r, bool bf, int np) {
     return {};
 }
 
-// Block list of order r: block (p, i) (lane offset d = dlo(p) + i) stacks
-// line 2d - p + r over line 2d - p + r + 1 (null outside 0..2r).
-std::vector<std::array<const double*, 2>> pair_blocks(int r, const double* cg) {
-    const int W = 2 * r + 1;
-    std::vector<std::array<const double*, 2>> out;
-    for (int p = 0; p < 2; ++p) {
-        const int dlo = -((r + 1 - p) / 2);
-        for (int i = 0; i <= r; ++i) {
-            std::array<const double*, 2> b{nullptr, nullptr};
+// Block list of order r, in their order along N (Pair::pos): block (p, i) (lane
+// offset d = dlo(p) + i) stacks line 2d - p + r over line 2d - p + r + 1 (null
+// outside 0..2r) and goes into output parity p.
+template <int R>
+std::vector<PairBlock> pair_blocks(const double* cg) {
+    using G = Pair<R>;
+    std::vector<PairBlock> out(G::NBLK);
+    for (int p = 0; p < 2; ++p)
+        for (int i = 0; i < G::NBP; ++i) {
+            PairBlock b{{nullptr, nullptr}, p};
             for (int e = 0; e < 2; ++e) {
-                const int a = 2 * (dlo + i) - p + r + e;
-                if (a >= 0 && a <= 2 * r) b[e] = cg + a * W;
+                const int a = 2 * (G::dlo(p) + i) - p + R + e;
+                if (a >= 0 && a <= 2 * R) b.line[e] = cg + a * (2 * R + 1);
             }
-            out.push_back(b);
+            out[G::pos(p, i)] = b;
         }
-    }
     return out;
+}
+
+std::vector<PairBlock> pair_blocks(int r, const double* cg) {
+    switch (r) {
+        case 1: return pair_blocks<1>(cg);
+        case 2: return pair_blocks<2>(cg);
+        case 3: return pair_blocks<3>(cg);
+        default: return pair_blocks<4>(cg);
+    }
 }
 
 // Row-parity view of a row-major grid with rows of ldx elements: rows parity,

@@ -6,7 +6,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <array>
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -274,10 +273,16 @@ inline float tf32_round(float x) {
 }
 
 
-// Banded operand of a block list: block j stacks, along K, the band of line
-// blocks[j][0] (K rows 0 .. kh-1) over the band of line blocks[j][1] (rows
-// kh .. 2kh-1); a null line contributes zeros.  Used when one TMEM lane holds
-// two input rows side by side along K.
+// One block of the 2D kernel's operand: the lines its even and odd input rows
+// are multiplied with (null: none) and the output row parity it goes into.
+struct PairBlock {
+    const double* line[2];
+    int parity;
+};
+
+// Banded operand of a block list: block j stacks, along K, the band of its
+// first line (K rows 0 .. kh-1) over the band of its second (rows kh ..
+// 2kh-1).  Used when one TMEM lane holds two input rows side by side along K.
 //
 // `cancel` (fused TF32x3 sweeps): the error of TF32x3 over many steps is a bias
 // of the field's amplitude from two sources, both cancelled here at no cost (a
@@ -300,8 +305,8 @@ inline float tf32_round(float x) {
 // short mantissas are exact, and nothing is truncated.
 constexpr double kTrunc = 0.7213475 * 0.5 / (1 << 23);   // E[2^e / x] / 2 ulp, x's mantissa log-uniform
 
-inline std::vector<unsigned char> pack_blocks(int r, const std::vector<std::array<const double*, 2>>& blocks, int nb,
-                                              int kh, bool bf, bool cancel, uint32_t* part_bytes) {
+inline std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& blocks, int nb, int kh,
+                                              bool bf, bool cancel, uint32_t* part_bytes) {
     const int nblk = (int)blocks.size(), N = nblk * nb, kw = 2 * kh;
     const int epc = bf ? 8 : 4;  // elements per 16-byte chunk
     const int es = bf ? 2 : 4;
@@ -311,17 +316,17 @@ inline std::vector<unsigned char> pack_blocks(int r, const std::vector<std::arra
     bool exact = true;
     for (const auto& b : blocks)
         for (int e = 0; e < 2; ++e)
-            for (int t = 0; b[e] && t < 2 * r + 1; ++t) exact = exact && (double)tf32_round((float)b[e][t]) == b[e][t];
+            for (int t = 0; b.line[e] && t < 2 * r + 1; ++t)
+                exact = exact && (double)tf32_round((float)b.line[e][t]) == b.line[e][t];
     cancel = cancel && !exact;
-    const int per_out = nblk / 2;                  // blocks summed into one output (parity j / per_out)
-    std::vector<double> carry(nb, 0.0);            // per output column
+    std::vector<double> carries(2 * nb, 0.0);      // per output parity and column
     for (int j = 0; j < nblk; ++j) {
-        if (j % per_out == 0) carry.assign(nb, 0.0);
         for (int q = 0; q < nb; ++q) {
+            double& carry = carries[blocks[j].parity * nb + q];
             // band entry of line e at window column kk: weight kk - q - (4 - r)
             auto weight = [&](int e, int kk) {
                 const int t = kk - q - (4 - r);
-                return blocks[j][e] && t >= 0 && t <= 2 * r ? blocks[j][e][t] : 0.0;
+                return blocks[j].line[e] && t >= 0 && t <= 2 * r ? blocks[j].line[e][t] : 0.0;
             };
             int adds = 0;                          // MMAs (8 columns each) that add to this block's column
             if (cancel)
@@ -341,9 +346,9 @@ inline std::vector<unsigned char> pack_blocks(int r, const std::vector<std::arra
                         if (step >= 0 && step != kk / 8) --adds;
                         step = kk / 8;
                         const double most = std::ldexp(std::fabs(w), -23);
-                        const double taken = std::min(std::max(carry[q], -most), most);
+                        const double taken = std::min(std::max(carry, -most), most);
                         rem = w * (1.0 + (adds - 0.5) * kTrunc) + taken;
-                        carry[q] -= taken;
+                        carry -= taken;
                     }
                     const int k = e * kh + kk;
                     const size_t off = ((size_t)(k / epc) * N + (size_t)(j * nb + q)) * 16 + (size_t)(k % epc) * es;
@@ -359,7 +364,7 @@ inline std::vector<unsigned char> pack_blocks(int r, const std::vector<std::arra
                             memcpy(&out[p * pb + off], &v, 4);
                         }
                     }
-                    if (cancel) carry[q] += rem;
+                    if (cancel) carry += rem;
                 }
                 if (step >= 0) --adds;
             }
