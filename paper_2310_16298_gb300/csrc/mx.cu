@@ -205,7 +205,7 @@ __host__ __device__ constexpr int d_sets(int a_cols, int n) {
 // is four adjacent columns of one row, the weights come from a table by the
 // point's distance class in y and x (one class when periodic).  The tiles
 // write only the rest of the grid, so the two need no order between them.
-// 8192^2, order 4: 32 thousand items over 152 warps cost 8 us of a 134 us
+// 8192^2, order 4: 32 thousand items over 152 warps cost 5 us of a 130 us
 // sweep (issue slots and the load/store pipe shared with the tiles' warps); a
 // second kernel over the strips cost 20.  Data comes through L2 (__ldcg): the
 // buffer was the output of an earlier sweep of the same stream.
@@ -242,6 +242,13 @@ __device__ __forceinline__ void boundary_strips(const MxArgs2D& a, int first, in
 #pragma unroll
         for (int q = 0; q < 4; ++q) cx[q] = strip_class(min(4 * g + q, a.nx - 1), a.nx, s);
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        // Input columns 4 g - 4 .. 4 g + 7: three groups, each wholly inside the
+        // grid or wholly outside it (then wrapped, or zero), unless the extent is
+        // no multiple of 4 and the item lies at an x face: then column by column.
+        // Predicated loads without branches, so that a chunk's are all in flight:
+        // with a branch per group the strips outlasted the tiles (8192^2 order 4
+        // periodic 135 us, now 130; 128^2 r = 1 2.5 us per step, now 2.2).
+        const bool whole = a.nx % 4 == 0 || (g > 0 && 4 * g + 8 <= a.nx);
         for (int d0 = 0; d0 < W; d0 += RB) {
             float v[RB][12];   // v[b][k] = column 4 g - 4 + k of row y - R + d0 + b
 #pragma unroll
@@ -251,23 +258,28 @@ __device__ __forceinline__ void boundary_strips(const MxArgs2D& a, int first, in
                 const bool use = d0 + b < W && (periodic || !wrap_y);
                 if (wrap_y) yy += yy < 0 ? a.ny : -a.ny;
                 const float* row = a.in + (int64_t)yy * a.ldx;
+                if (whole) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int x = 4 * (g - 1 + k);
-                    float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    if (use && x >= 0 && x + 3 < a.nx) {
-                        u = __ldcg(reinterpret_cast<const float4*>(row + x));
-                    } else if (use) {   // group across the x face: column by column
-                        auto at = [&](int c) {
-                            if (c >= 0 && c < a.nx) return __ldcg(row + c);
-                            return periodic ? __ldcg(row + (c < 0 ? c + a.nx : c - a.nx)) : 0.0f;
-                        };
-                        u = make_float4(at(x), at(x + 1), at(x + 2), at(x + 3));
+                    for (int k = 0; k < 3; ++k) {
+                        int x = 4 * (g - 1 + k);
+                        const bool in = x >= 0 && x < a.nx;
+                        x += in ? 0 : x < 0 ? a.nx : -a.nx;
+                        float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        if (use && (in || periodic)) u = __ldcg(reinterpret_cast<const float4*>(row + x));
+                        v[b][4 * k] = u.x;
+                        v[b][4 * k + 1] = u.y;
+                        v[b][4 * k + 2] = u.z;
+                        v[b][4 * k + 3] = u.w;
                     }
-                    v[b][4 * k] = u.x;
-                    v[b][4 * k + 1] = u.y;
-                    v[b][4 * k + 2] = u.z;
-                    v[b][4 * k + 3] = u.w;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 12; ++k) {
+                        int x = 4 * g - 4 + k;
+                        const bool in = x >= 0 && x < a.nx;
+                        x += in ? 0 : x < 0 ? a.nx : -a.nx;
+                        v[b][k] = 0.0f;
+                        if (use && (in || periodic)) v[b][k] = __ldcg(row + x);
+                    }
                 }
             }
 #pragma unroll
