@@ -231,7 +231,7 @@ def oracle_baseline(p, field, max_seconds=20.0):
 
 # Tile periods of the matrixized kernels along each axis (slowest first):
 # 2D tiles are 4 lane quarters of 2 (32 - 2 ceil(r/2)) rows by 2 items of 16
-# columns; 3D work units are 32-plane chunks by 4 quarters of 32 - 2r rows by
+# columns; 3D work units are chunks of up to 32 planes by 4 columns of 32 - 2r rows by
 # 16 or 32 columns.  Seams between them are sampled on purpose.
 def tile_periods(ndim, r):
     if ndim == 2:
@@ -512,7 +512,7 @@ def run_ablation(args):
             stream.synchronize()
             ms = float(np.median([a_.elapsed_time(b_) for a_, b_ in ev]))
             tile_n = plan.info["tile_n"]
-            units = -(-side // up) * -(-side // 120) * -(-side // tile_n)
+            units = -(-side // up) * -(-(-(-side // 30) * -(-side // tile_n)) // 4)
             rows.append({"kind": kind, "unit_planes": up, "input_planes_per_output_plane": (up + 2) / up,
                          "units": units, "ms_per_sweep": ms, "gstencil_s": x.numel() / ms / 1e6})
             plan.close()

@@ -5,12 +5,13 @@
 // of width r*tb in shared memory, performs tb sub-steps there (the valid
 // region shrinks by r per sub-step; with a zero Dirichlet boundary, points
 // outside the domain are reset to 0 after every sub-step), and writes the
-// tile once.  Each thread computes a strip of RS outputs along the slowest
-// axis, reusing every loaded shared-memory row for all outputs it feeds.
+// tile once.  Each thread computes blocks of 4 x 4 outputs (2D FP32) or strips
+// of outputs along the slowest axis, reusing every loaded shared-memory row
+// for all outputs it feeds.
 //
 // Single grids run persistent kernels that stage their tiles with TMA:
 //  * 2D: each CTA walks its tiles through a ring of NST shared-memory stages
-//    (four for FP32, two for FP64), the next tiles' halo blocks loading (one
+//    (two or three), the next tiles' halo blocks loading (one
 //    cp.async.bulk.tensor each, zero fill outside the grid = the Dirichlet
 //    halo) while the current one computes.
 //  * 3D (one step per launch): a work unit is a column of output planes; the

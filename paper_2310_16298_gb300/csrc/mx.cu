@@ -33,8 +33,11 @@
 // last CTA to finish), so SMs that run faster take more tiles.
 //
 // Boundaries: rows and columns outside the grid are TMA's out-of-bounds zero
-// fill (the zero Dirichlet halo); with a periodic boundary the terms that
-// wrap are added afterwards by the edge kernel (edges.cu).
+// fill (the zero Dirichlet halo).  With a periodic boundary, or when a sweep
+// advances several steps (R is then the order of the composed stencil), the
+// points near the faces are boundary strips, computed beside the tiles; on
+// small grids and in plain precisions the periodic boundary's wrapped terms
+// are added afterwards by the edge kernel (edges.cu).
 //
 // Roles (one persistent CTA per SM, warp specialised):
 //  * warp 0: TMA producer.  A tile is 4 lane quarters x 64 input rows; each
@@ -50,6 +53,7 @@
 //  * warps 10..17: epilogue warps, one per (quarter, output parity): tensor
 //    memory -> shuffles -> swizzled smem -> TMA store through the output
 //    row-parity tensor map.
+//  * warp 19: boundary strips, straight from and to global memory.
 // Two or three accumulator sets and A stages (as many as tensor memory
 // holds) overlap split, MMA and epilogue; every wait is bounded
 // (a timeout sets a host-visible error word, drains copies in flight and
