@@ -125,6 +125,7 @@ stencil_status upload_tables(int n, const stencil_plan_t* plans, const Schedule&
     cudaError_t e = cudaMalloc(&d, total);
     if (e != cudaSuccess) return fail(STENCIL_ENOMEM, "batch tables");
     e = cudaMemcpy(d, host.data(), total, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // staged copies may end after the call
     if (e != cudaSuccess) {
         cudaFree(d);
         return cuda_fail(e, "batch table upload");

@@ -715,6 +715,10 @@ stencil_status mx3d_plan_build(const MxRequest& q, MxPlan* p, std::string* why) 
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&st->err_dev, st->err_host, 0);
     if (e == cudaSuccess) e = cudaMalloc(&st->sched, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(st->sched, 0, 2 * sizeof(int));
+    // The upload and the memset may still be under way, and the sweeps run on
+    // streams that do not wait for the legacy stream: with other work on the GPU a
+    // first sweep could start before its unit counter was zero.
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&st->num_sms, cudaDevAttrMultiProcessorCount, dev);
