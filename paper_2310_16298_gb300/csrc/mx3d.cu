@@ -619,10 +619,12 @@ bool encode_out_map_3d(CUtensorMap* map, float* base, int nz, int ny, int nx, in
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+constexpr size_t kSchedBytes3 = 256;   // of the operand buffer: the unit counters
+
 struct Mx3State {
     unsigned int* err_host = nullptr;
     unsigned int* err_dev = nullptr;
-    int* sched = nullptr;  // device unit counter pair (zero between launches)
+    int* sched = nullptr;  // device unit counter pair (in the operand buffer; zero between launches)
     int num_sms = 0;
     int nb = 16;
     int in_w = 24;
@@ -690,6 +692,9 @@ stencil_status mx3d_plan_build(const MxRequest& q, MxPlan* p, std::string* why) 
     p->n_lines = L;
     p->n_scalar = hyb ? 4 * r : 0;
     p->cover = hyb ? STENCIL_COVER_HYBRID : STENCIL_COVER_PARALLEL;
+    // one buffer: the unit counter pair (zero), then the banded operands
+    const size_t ops_bytes = ops.size();
+    ops.insert(ops.begin(), kSchedBytes3, 0);
     p->operand_bytes = ops.size();
     cudaError_t e = cudaMalloc(&p->d_operands, p->operand_bytes);
     if (e != cudaSuccess) {
@@ -709,15 +714,15 @@ stencil_status mx3d_plan_build(const MxRequest& q, MxPlan* p, std::string* why) 
             st->sw[k] = (float)q.cg[((size_t)o * W + r) * W + r];            // z offset o
             st->sw[2 * r + k] = (float)q.cg[((size_t)r * W + o) * W + r];    // y offset o
         }
-    st->bop_bytes = (uint32_t)p->operand_bytes;
+    st->bop_bytes = (uint32_t)ops_bytes;
+    st->sched = (int*)p->d_operands;
     st->bpart_bytes = bpart;
     if (e == cudaSuccess) e = cudaHostAlloc((void**)&st->err_host, sizeof(unsigned int), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&st->err_dev, st->err_host, 0);
-    if (e == cudaSuccess) e = cudaMalloc(&st->sched, 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(st->sched, 0, 2 * sizeof(int));
-    // The upload and the memset may still be under way, and the sweeps run on
-    // streams that do not wait for the legacy stream: with other work on the GPU a
-    // first sweep could start before its unit counter was zero.
+    // The upload may still be under way, and the sweeps run on streams that do not
+    // wait for the legacy stream: with other work on the GPU a first sweep could
+    // start before its unit counter was zero.  (Part of the upload, not a memset:
+    // that waits for a free SM.)
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -742,7 +747,6 @@ void mx3d_plan_free(MxPlan* p) {
     Mx3State* st = (Mx3State*)p->tmap_storage;
     if (st) {
         if (st->err_host) cudaFreeHost(st->err_host);
-        if (st->sched) cudaFree(st->sched);
         delete st;
     }
     p->tmap_storage = nullptr;
@@ -763,7 +767,7 @@ cudaError_t mx3d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     MxArgs3D a;
     memset(&a, 0, sizeof(a));
     a.bc = p.bc;
-    a.bops = p.d_operands;
+    a.bops = (const unsigned char*)p.d_operands + kSchedBytes3;
     a.err = st->err_dev;
     a.sched = st->sched;
     a.nz = nz;
