@@ -1028,6 +1028,21 @@ size_t tile2_smem_bytes(int r, int tb, int ty, int tx) {
     return (size_t)((tb > 1 ? 2 : 1) * (ty + 2 * H) + kRS) * (tx + 2 * H) * sizeof(T);
 }
 
+int max_smem_optin() {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return v;
+}
+
+// Let a kernel take as much dynamic shared memory as the device allows.  The
+// limit belongs to the kernel, and plans and launches of different depth share
+// one: set to what one of them needs, it would fall below what another needs.
+template <typename K>
+cudaError_t allow_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem_optin());
+}
+
 template <typename T, int R, bool STAR>
 cudaError_t launch2d_tiles(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
     constexpr int NC = ipow(2 * R + 1, 2);
@@ -1035,7 +1050,7 @@ cudaError_t launch2d_tiles(const GatherProblem& p, const void* in, void* out, in
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
     const size_t smem = tile2_smem_bytes<T>(R, tb, k2TY, k2TX);
     auto kern = gather2d_kernel<T, R, STAR, k2BY, k2TX, k2TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p.n[1] + k2TX - 1) / k2TX), (unsigned)((p.n[0] + k2TY - 1) / k2TY));
     kern<<<grid, dim3(kBX, k2BY), smem, s>>>((const T*)in, (T*)out, p.n[0], p.n[1], p.ldx, p.bc, tb, cf);
@@ -1049,19 +1064,12 @@ cudaError_t launch3d_tiles(const GatherProblem& p, const void* in, void* out, in
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
     const size_t smem = gather_smem_bytes_t<T>(3, R, tb);
     auto kern = gather3d_kernel<T, R, STAR, k3BY, k3TX, k3TY, k3TZ>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p.n[2] + k3TX - 1) / k3TX), (unsigned)((p.n[1] + k3TY - 1) / k3TY),
               (unsigned)((p.n[0] + k3TZ - 1) / k3TZ));
     kern<<<grid, dim3(kBX, k3BY), smem, s>>>((const T*)in, (T*)out, p.n[0], p.n[1], p.n[2], p.ldx, p.bc, tb, cf);
     return cudaGetLastError();
-}
-
-int max_smem_optin() {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return v;
 }
 
 int sm_count() {
@@ -1104,7 +1112,7 @@ cudaError_t tuned_for(const GatherProblem& p, K kern, int threads, size_t smem, 
         *t = *p.tuned;
         if (t->per_sm[tb] > 0) return cudaSuccess;
     }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     t->sms = sm_count();
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t->per_sm[tb], kern, threads, smem);
@@ -1232,7 +1240,7 @@ cudaError_t launch_batch(const BatchProblem* probs, int nprob, int total_tiles, 
     const size_t smem = batch_smem_bytes_t<T>(R, max_tb, S);
     constexpr int BY = sizeof(T) == 4 ? kBatchBY[S] : k2BY;
     auto kern = gather2d_batch_kernel<T, R, STAR, BY, kBatchTX[S], kBatchTY[S]>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     if (grid <= 0) {
         int dev = 0, sms = 0, per = 0;
