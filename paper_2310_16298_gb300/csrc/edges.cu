@@ -69,7 +69,7 @@ __device__ __forceinline__ int wrap1(int i, int n) { return i < 0 ? i + n : (i >
 // issued before the first is used.  The point's own output value is loaded
 // first.  One copy of the chunk code serves all segments (the kernel is short
 // lived, so its instruction footprint is part of its latency).
-__global__ void __launch_bounds__(128) periodic_edges_kernel(const float* __restrict__ in, float* __restrict__ out,
+__global__ void __launch_bounds__(128) periodic_edges_kernel(const float* in, float* out,
                                                              int nz, int ny, int nx, int64_t ldx, int r,
                                                              const __grid_constant__ EdgeTable tab) {
     constexpr int C = 8;
@@ -80,7 +80,10 @@ __global__ void __launch_bounds__(128) periodic_edges_kernel(const float* __rest
     const int z = blockIdx.y;
     // launched as a programmatic dependent of the tensor-core kernel: let the
     // next sweep's kernel start its set-up, then wait until the tensor-core
-    // grid has completed and its writes are visible
+    // grid has completed and its writes are visible.  A small grid's tensor-core
+    // kernel lets this one start at once, so it may be resident while the
+    // kernels before that still write `in`: the fields are read through L2
+    // (__ldcg), never through the read-only path or lines that L1 kept.
     ptx::launch_dependents();
     ptx::grid_dependency_wait();
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < per_plane; p += gridDim.x * blockDim.x) {
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(128) periodic_edges_kernel(const float* __rest
             x = nx <= 2 * r ? c : (c < r ? c : nx - 2 * r + c);
         }
         float* o = out + ((int64_t)z * ny + y) * ldx + x;
-        const float o0 = *o;
+        const float o0 = __ldcg(o);
         const bool y_edge = y < r || y >= ny - r;
         const bool x_edge = x < r || x >= nx - r;
         float acc = 0.0f;
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(128) periodic_edges_kernel(const float* __rest
                     // x segments skip the terms the y segments took
                     const bool use = c + k < t1 && !(by_x && y_edge && (yy < 0 || yy >= ny));
                     const int64_t off = ((int64_t)wrap1(z + e.dz, nz) * ny + wrap1(yy, ny)) * ldx + wrap1(x + e.dx, nx);
-                    v[k] = use ? __ldg(in + off) : 0.0f;
+                    v[k] = use ? __ldcg(in + off) : 0.0f;
                 }
 #pragma unroll
                 for (int k = 0; k < C; ++k) acc = fmaf(terms[min(c + k, kMaxEdgeTerms - 1)].w, v[k], acc);
