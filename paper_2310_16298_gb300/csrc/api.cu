@@ -41,7 +41,7 @@ stencil_status cuda_fail(cudaError_t e, const char* what) {
 
 const std::string& last_error_string() { return g_err; }
 
-GatherProblem gather_problem(const stencil_plan_s* p) {
+GatherProblem gather_problem(const stencil_plan_s* p, int* sched) {
     GatherProblem g;
     g.ndim = p->ndim;
     for (int d = 0; d < 3; ++d) g.n[d] = p->n[d];
@@ -53,16 +53,104 @@ GatherProblem gather_problem(const stencil_plan_s* p) {
     g.err = p->err_dev;
     g.ldx = p->ldx;
     g.tuned = p->is_tuned ? &p->tuned : nullptr;
-    g.sched = p->gather_sched;
+    g.sched = sched;
     return g;
 }
 
-// One sweep of depth `tb` from src to dst.
-cudaError_t run_sweep(const stencil_plan_s* p, const void* src, void* dst, int tb, cudaStream_t s) {
+// One sweep of depth `tb` from src to dst; `sched`: the gather kernels' tile counter pair.
+cudaError_t run_sweep(const stencil_plan_s* p, const void* src, void* dst, int tb, int* sched, cudaStream_t s) {
     if (p->impl == STENCIL_IMPL_MATRIXIZED) return mx_sweep(*p->mx, src, dst, tb, s);
-    GatherProblem g = gather_problem(p);
+    GatherProblem g = gather_problem(p, sched);
     return gather_sweep(g, src, dst, tb, s);
 }
+
+namespace {
+
+// Tile counter pairs of the gather plans: zero-initialised device memory of the
+// library (one allocation, copy or memset less per plan).  Every launch leaves
+// its pair at zero, so launches that cannot overlap may share one; those that
+// find none run with fixed tile shares.
+constexpr int kCounters = 1024;
+__device__ int g_counters[kCounters][2];
+struct Counters {
+    int* base = nullptr;
+    int* noalloc = nullptr;    // of the sweeps through stencil_apply_noalloc's array
+    std::vector<int> free;
+};
+std::mutex g_counters_mu;
+std::map<int, Counters> g_counters_of;   // by device
+
+int* take(Counters& c) {
+    if (!c.base) {
+        void* q = nullptr;
+        if (cudaGetSymbolAddress(&q, g_counters) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c.base = (int*)q;
+        for (int i = kCounters - 1; i >= 0; --i) c.free.push_back(i);
+    }
+    if (c.free.empty()) return nullptr;
+    const int i = c.free.back();
+    c.free.pop_back();
+    return c.base + 2 * i;
+}
+
+int* counter_take(int device) {
+    std::lock_guard<std::mutex> lk(g_counters_mu);
+    return take(g_counters_of[device]);
+}
+
+void counter_give(int device, int* counter) {
+    if (!counter) return;
+    std::lock_guard<std::mutex> lk(g_counters_mu);
+    Counters& c = g_counters_of[device];
+    c.free.push_back((int)(counter - c.base) / 2);
+}
+
+// Which launches may share a pair.  Applies that go through a scratch grid
+// are ordered by the caller (they would race on the grid), so the grid's pair
+// serves them all, in captured graphs too.  A single sweep from d_in to d_out
+// touches no scratch grid, and such applies of one plan may overlap: those of
+// one stream cannot, and share a pair; beyond kStreamCounters streams, and in
+// a graph, which may be replayed on any stream, they take fixed shares.
+int* counter_of_scratch(const stencil_plan_s* p, const void* scratch) {
+    if (scratch == p->scratch) return p->gather_sched;
+    std::lock_guard<std::mutex> lk(g_counters_mu);
+    Counters& c = g_counters_of[p->device];
+    if (!c.noalloc) c.noalloc = take(c);
+    return c.noalloc;
+}
+
+int* counter_of_stream(const stencil_plan_s* p, cudaStream_t s) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) return nullptr;
+    // asking for the id ends a capture: not asked of a capturing stream, and in
+    // relaxed mode, so that it is no matter to one that another thread runs
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (e == cudaSuccess) e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+        e = cudaStreamGetId(s, &id);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    std::lock_guard<std::mutex> lk(p->stream_mu);
+    for (auto& k : p->stream_sched) {
+        if (!k.counter) {
+            k.id = id;
+            k.counter = counter_take(p->device);
+        }
+        if (k.counter && k.id == id) return k.counter;
+    }
+    return nullptr;
+}
+
+}  // namespace
 
 // Time loop (Sec. 2.2: two grid copies used alternately).  The copies are the
 // caller's output and the plan's scratch grid, ordered so that the last
@@ -80,6 +168,7 @@ stencil_status time_loop(const stencil_plan_s* p, const void* d_in, void* d_out,
                          cudaStream_t s, void* scratch) {
     if (steps > 0 && p->repack) {
         // the field goes into the plan's padded grids, is advanced there and comes back
+        // (tensor-core plans only)
         void* g[2] = {p->pad, p->scratch};
         cudaError_t e = repack_copy(p, g[0], p->ldx, d_in, p->pitch, s);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy2DAsync");
@@ -87,7 +176,7 @@ stencil_status time_loop(const stencil_plan_s* p, const void* d_in, void* d_out,
         const int64_t nsweep = (steps + tb - 1) / tb;
         for (int64_t k = 0; k < nsweep; ++k) {
             const int depth = (int)((k == nsweep - 1) ? (steps - (nsweep - 1) * tb) : tb);
-            e = run_sweep(p, g[k & 1], g[(k + 1) & 1], depth, s);
+            e = run_sweep(p, g[k & 1], g[(k + 1) & 1], depth, nullptr, s);
             if (e != cudaSuccess) return cuda_fail(e, "stencil sweep launch");
         }
         e = repack_copy(p, d_out, p->pitch, g[nsweep & 1], p->ldx, s);
@@ -109,11 +198,14 @@ stencil_status time_loop(const stencil_plan_s* p, const void* d_in, void* d_out,
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync");
         src = scratch;
     }
+    int* sched = nullptr;
+    if (p->impl == STENCIL_IMPL_GATHER && p->ndim == 2 && !p->f64)   // the kernels that claim tiles
+        sched = nsweep > 1 || src == scratch ? counter_of_scratch(p, scratch) : counter_of_stream(p, s);
     for (int64_t k = 0; k < nsweep; ++k) {
         const int64_t left = nsweep - 1 - k;  // sweeps after this one
         void* dst = (left & 1) ? scratch : d_out;
         const int depth = (int)((k == nsweep - 1) ? (steps - (nsweep - 1) * tb) : tb);
-        cudaError_t e = run_sweep(p, src, dst, depth, s);
+        cudaError_t e = run_sweep(p, src, dst, depth, sched, s);
         if (e != cudaSuccess) return cuda_fail(e, "stencil sweep launch");
         src = dst;
     }
@@ -206,44 +298,6 @@ stencil_status ticket_done(uint64_t ticket, const Ticket& t, cudaError_t e) {
 // =================================================================== plans
 namespace {
 
-// Tile counter pairs of the gather plans: zero-initialised device memory of the
-// library (one allocation, copy or memset less per plan), handed out per plan
-// and returned with it.  Every launch leaves its pair at zero.  A plan that
-// finds none left runs with fixed tile shares.
-constexpr int kCounters = 1024;
-__device__ int g_counters[kCounters][2];
-struct Counters {
-    int* base = nullptr;
-    std::vector<int> free;
-};
-std::mutex g_counters_mu;
-std::map<int, Counters> g_counters_of;   // by device
-
-int* counter_take(int device) {
-    std::lock_guard<std::mutex> lk(g_counters_mu);
-    Counters& c = g_counters_of[device];
-    if (!c.base) {
-        void* q = nullptr;
-        if (cudaGetSymbolAddress(&q, g_counters) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        c.base = (int*)q;
-        for (int i = kCounters - 1; i >= 0; --i) c.free.push_back(i);
-    }
-    if (c.free.empty()) return nullptr;
-    const int i = c.free.back();
-    c.free.pop_back();
-    return c.base + 2 * i;
-}
-
-void counter_give(int device, int* counter) {
-    if (!counter) return;
-    std::lock_guard<std::mutex> lk(g_counters_mu);
-    Counters& c = g_counters_of[device];
-    c.free.push_back((int)(counter - c.base) / 2);
-}
-
 // Free everything a plan (complete or half-built) owns.
 void plan_free(stencil_plan_s* p) {
     if (!p) return;
@@ -251,8 +305,11 @@ void plan_free(stencil_plan_s* p) {
     if (p->scratch) cudaFree(p->scratch);
     if (p->staging) cudaFree(p->staging);
     if (p->pad) cudaFree(p->pad);
-    // (after an aborted kernel the pair may not be zero: it is not handed out again)
-    if (!p->err_host || *(volatile unsigned int*)p->err_host == 0) counter_give(p->device, p->gather_sched);
+    // (after an aborted kernel the pairs may not be zero: they are not handed out again)
+    if (!p->err_host || *(volatile unsigned int*)p->err_host == 0) {
+        counter_give(p->device, p->gather_sched);
+        for (auto& k : p->stream_sched) counter_give(p->device, k.counter);
+    }
     if (p->err_host) cudaFreeHost(p->err_host);
     if (p->stream) cudaStreamDestroy(p->stream);
     if (p->mx) {
@@ -463,7 +520,7 @@ extern "C" stencil_status stencil_plan_create(stencil_plan_t* out, int ndim, con
         if (e != cudaSuccess) return cuda_fail(e, "error word");
         *p->err_host = 0;
         p->tb = o.tb > 0 ? o.tb : 1;
-        GatherProblem g = gather_problem(p.get());
+        GatherProblem g = gather_problem(p.get(), nullptr);
         int max_smem = 0;
         e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");

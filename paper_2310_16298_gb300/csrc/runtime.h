@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -42,7 +43,16 @@ struct stencil_plan_s {
     void* staging = nullptr;        // device grid of stencil_apply_host (allocated on first use)
     unsigned int* err_host = nullptr;  // host-mapped error word of the gather kernels' bounded waits
     unsigned int* err_dev = nullptr;
-    int* gather_sched = nullptr;    // tile counter pair of the gather kernels (null: none was left)
+    // Tile counter pairs of the gather kernels (null: none was left, or not yet taken): of the sweeps
+    // that go through the scratch grid, and of single sweeps by stream.
+    int* gather_sched = nullptr;
+    struct StreamCounter {
+        unsigned long long id = 0;   // cudaStreamGetId: never reused
+        int* counter = nullptr;
+    };
+    static constexpr int kStreamCounters = 4;
+    mutable StreamCounter stream_sched[kStreamCounters];
+    mutable std::mutex stream_mu;
     stx::GatherTuned tuned;         // launch shapes of the gather kernels
     bool is_tuned = false;
 };
@@ -55,8 +65,6 @@ stencil_status fail(stencil_status st, const std::string& msg);
 stencil_status cuda_fail(cudaError_t e, const char* what);
 const std::string& last_error_string();
 
-GatherProblem gather_problem(const stencil_plan_s* p);
-cudaError_t run_sweep(const stencil_plan_s* p, const void* src, void* dst, int tb, cudaStream_t s);
 // Advance d_in by `steps` into d_out on stream s, ping-ponging through `scratch`.
 stencil_status time_loop(const stencil_plan_s* p, const void* d_in, void* d_out, int64_t steps, cudaStream_t s,
                          void* scratch);
