@@ -282,6 +282,7 @@ void worker_loop(stencil_server_s* S) {
                 }
             }
             cudaStream_t s = S->streams[q->stream];
+            cudaError_t e = cudaSuccess;
             if (q->done_steps < q->steps) {
                 // whole sweeps (a plan may advance several steps per sweep), so that
                 // the steps fuse as in one apply of all of them
@@ -298,12 +299,21 @@ void worker_loop(stencil_server_s* S) {
                 S->issued += 1;
             } else {
                 // all steps issued: bring the result home
-                cudaMemcpyAsync(q->result, q->grid, q->grid_bytes, cudaMemcpyDeviceToHost, s);
+                e = cudaMemcpyAsync(q->result, q->grid, q->grid_bytes, cudaMemcpyDeviceToHost, s);
                 q->draining = true;
             }
-            cudaEventRecord(q->ev, s);
-            q->in_flight = true;
+            if (e == cudaSuccess) e = cudaEventRecord(q->ev, s);
             progressed = true;
+            if (e != cudaSuccess) {
+                // without the copy its buffer holds an earlier request's result, and
+                // without the event nothing says when the copy has ended
+                cudaStreamSynchronize(s);
+                q->error = STENCIL_ECUDA;
+                q->message = std::string("request work: ") + cudaGetErrorString(e);
+                finished.push_back(q);
+                continue;
+            }
+            q->in_flight = true;
         }
         if (!finished.empty()) {
             std::lock_guard<std::mutex> lk(S->mu);
