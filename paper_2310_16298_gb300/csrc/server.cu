@@ -129,7 +129,18 @@ cudaError_t pinned_take(stencil_server_s* S, size_t bytes, void** out, size_t* g
         }
     }
     *got = bytes;
-    return cudaMallocHost(out, bytes);
+    cudaError_t e = cudaMallocHost(out, bytes);
+    if (e != cudaSuccess) {   // kept buffers that do not fit may hold what is missing
+        cudaGetLastError();
+        {
+            std::lock_guard<std::mutex> lk(S->pinned_mu);
+            for (auto& kv : S->pinned) cudaFreeHost(kv.second);
+            S->pinned.clear();
+            S->pinned_bytes = 0;
+        }
+        e = cudaMallocHost(out, bytes);
+    }
+    return e;
 }
 
 void pinned_give(stencil_server_s* S, void* buf, size_t bytes) {

@@ -15,7 +15,7 @@
 static std::atomic<int> fail_d2h{0}, fail_record{0};   // > 0: the next so many calls fail
 static std::mutex mu;
 static std::map<void*, size_t> pinned;
-static size_t pinned_now = 0;
+static size_t pinned_now = 0, pinned_most = (size_t)1 << 40;
 
 extern "C" {
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
@@ -42,6 +42,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, 
 }
 cudaError_t cudaMallocHost(void** p, size_t n) {
     std::lock_guard<std::mutex> lk(mu);
+    if (pinned_now + n > pinned_most) return cudaErrorMemoryAllocation;
     *p = malloc(n);
     pinned[*p] = n;
     pinned_now += n;
@@ -111,7 +112,8 @@ int main(int argc, char** argv) {
     if (solve(s, 64, 5.0f, &v) != STENCIL_OK || v != 15.0f) return 3;
     if (what == "copy") fail_d2h = 1;
     if (what == "record") fail_record = 1;
-    const int st = solve(s, 64, 7.0f, &v);
+    if (what == "pinned") pinned_most = 140 << 10;   // the kept buffer has 64 KiB, the next result needs 128
+    const int st = solve(s, what == "pinned" ? 130 : 64, 7.0f, &v);
     printf("%d", st);
     if (st == STENCIL_OK) printf(" %g", v);
     // the server goes on

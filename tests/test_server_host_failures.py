@@ -40,3 +40,8 @@ def test_requests_without_failures(serve):
 def test_a_failed_result_copy_fails_the_request(serve, call):
     """Not OK with the result that an earlier request left in the kept buffer."""
     assert serve(call) == [str(sx.ECUDA)]
+
+
+def test_kept_buffers_make_room_for_a_result(serve):
+    """Pinned memory runs out while the server keeps a buffer that is too small."""
+    assert serve("pinned") == [str(sx.OK), "17"]
