@@ -25,6 +25,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "mxutil.cuh"
@@ -213,15 +215,17 @@ __device__ __forceinline__ void last_substep_f32(const float* src, float* __rest
 // either boundary) and advanced by tb steps; buffers a and b ping-pong.  A
 // grid without 16-byte rows gets its outputs through shared memory: written
 // as blocks, four 4-byte stores 16 bytes apart per lane would touch every
-// sector four times.
-template <int R, bool STAR, int TY, int TX>
+// sector four times.  WIDE: the last tiles of a row reach past column 2^31 (a
+// template parameter: 64-bit columns in every tile cost up to 5%, 1021 x 1533).
+template <int R, bool STAR, int TY, int TX, bool WIDE = false>
 __device__ __forceinline__ void tile2_f32(const float* __restrict__ in, float* __restrict__ out, int ny, int nx,
                                           int64_t ldx, int bc, int tb, const Coeffs<float, ipow(2 * R + 1, 2)>& cf,
                                           int y0, int x0, float* a, float* b, int tid, int nthreads) {
     const TileGeom g(R, tb, TY, TX);
     const int gy0 = y0 - g.H, gx0 = x0 - g.HX;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
-    const bool inside = gy0 >= 0 && gy0 + g.SY <= ny && gx0 >= 0 && gx0 + g.SX <= nx;
+    const auto gxl = (std::conditional_t<WIDE, int64_t, int>)gx0;
+    const bool inside = gy0 >= 0 && gy0 + g.SY <= ny && gx0 >= 0 && gxl + g.SX <= nx;
     const bool vec = ldx % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
     for (int sy = warp; sy < g.SY; sy += nwarps) {
         float* d = a + sy * g.SX;
@@ -233,7 +237,7 @@ __device__ __forceinline__ void tile2_f32(const float* __restrict__ in, float* _
             for (int sx = lane; sx < g.SX; sx += 32) cp_async_elem(d + sx, s + sx);
         } else {
             for (int sx = lane; sx < g.SX; sx += 32) {
-                const float* s = src2(in, gy0 + sy, gx0 + sx, ny, nx, ldx, bc);
+                const float* s = src2(in, gy0 + sy, gxl + sx, ny, nx, ldx, bc);
                 if (s) cp_async_elem(d + sx, s);
                 else d[sx] = 0.0f;
             }
@@ -348,15 +352,16 @@ __device__ __forceinline__ void gather2d_tile(const T* __restrict__ in, T* __res
     }
 }
 
-template <typename T, int R, bool STAR, int BY, int TX, int TY>
+template <typename T, int R, bool STAR, int BY, int TX, int TY, bool WIDE>
 __global__ void __launch_bounds__(kBX * BY)
 gather2d_kernel(const T* __restrict__ in, T* __restrict__ out, int64_t ny, int64_t nx, int64_t ldx, int bc,
                 int tb, Coeffs<T, ipow(2 * R + 1, 2)> cf) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if constexpr (sizeof(T) == 4) {
         float* a = reinterpret_cast<float*>(smem_raw) + kLeadElems;
-        tile2_f32<R, STAR, TY, TX>(in, out, (int)ny, (int)nx, ldx, bc, tb, cf, (int)blockIdx.y * TY, (int)blockIdx.x * TX,
-                                   a, a + TileGeom(R, tb, TY, TX).elems(), threadIdx.y * kBX + threadIdx.x, kBX * BY);
+        tile2_f32<R, STAR, TY, TX, WIDE>(in, out, (int)ny, (int)nx, ldx, bc, tb, cf, (int)blockIdx.y * TY,
+                                         (int)blockIdx.x * TX, a, a + TileGeom(R, tb, TY, TX).elems(),
+                                         threadIdx.y * kBX + threadIdx.x, kBX * BY);
     } else {
         gather2d_tile<T, R, STAR, BY, TX, TY>(in, out, ny, nx, ldx, bc, tb, cf, (int64_t)blockIdx.y * TY,
                                               (int64_t)blockIdx.x * TX, reinterpret_cast<T*>(smem_raw));
@@ -1049,7 +1054,9 @@ cudaError_t launch2d_tiles(const GatherProblem& p, const void* in, void* out, in
     Coeffs<T, NC> cf;
     for (int i = 0; i < NC; ++i) cf.c[i] = (T)p.cg[i];
     const size_t smem = tile2_smem_bytes<T>(R, tb, k2TY, k2TX);
-    auto kern = gather2d_kernel<T, R, STAR, k2BY, k2TX, k2TY>;
+    constexpr bool F32 = sizeof(T) == 4;   // (FP64 tiles compute all columns in 64 bits)
+    auto kern = F32 && p.n[1] > INT32_MAX - 512 ? gather2d_kernel<T, R, STAR, k2BY, k2TX, k2TY, F32>
+                                                : gather2d_kernel<T, R, STAR, k2BY, k2TX, k2TY, false>;
     cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p.n[1] + k2TX - 1) / k2TX), (unsigned)((p.n[0] + k2TY - 1) / k2TY));
