@@ -110,8 +110,9 @@ typedef struct {
     int32_t tb;       /* time steps fused per sweep (temporal blocking); 0 = library choice: 1,
                          or, for 2D matrixized plans of order 1 / 2 in TF32X3 or BF16X3 with
                          extents of at least 96, up to 4 / 2 steps evaluated as one step of
-                         the composed stencil.  An apply of n steps then runs n / tb whole
-                         sweeps and a shorter last one                                       */
+                         the composed stencil (not where a short or narrow grid's faces would
+                         cost more than that saves).  An apply of n steps then runs n / tb
+                         whole sweeps and a shorter last one                                 */
     int32_t cover;    /* stencil_cover; default AUTO (EINVAL when out of range)                 */
     int32_t pitch;    /* row stride of the grids, in elements (0 = packed rows); >= the
                          contiguous extent and a multiple of 16 bytes, else EINVAL.  Padding
@@ -139,11 +140,12 @@ typedef struct {
                              bounded wait (or stencil_plan_raise_error set bits)        */
     int32_t cover;        /* stencil_cover the matrixized kernel runs (0 for GATHER)    */
     int32_t kernels_per_sweep; /* kernel launches per sweep: 2 for MATRIXIZED plans with
-                             a periodic boundary, except 2D ones of FP32-class
-                             arithmetic with extents of at least 96 (the tensor-core kernel, whose TMA
+                             a periodic boundary (the tensor-core kernel, whose TMA
                              loads see zeros outside the grid in x and y, then a
-                             kernel over the boundary strips that adds the wrapped
-                             terms), else 1                                             */
+                             kernel over the points at the faces that adds the wrapped
+                             terms), except 2D ones of FP32-class arithmetic whose
+                             kernel computes those points itself (extents of at least
+                             96, not too short or narrow); else 1                       */
 } stencil_plan_info_t;
 
 /* ---------------------------------------------------------------------------

@@ -97,7 +97,7 @@ constexpr int kMma2Warp = 2 + kSplitWarps + kEpiWarps;   // second MMA issuer
 constexpr int kStripWarp = kMma2Warp + 1;                // boundary strips
 constexpr int kThreads = 32 * (kStripWarp + 1);
 constexpr int kMaxDepth = 4;            // time steps one sweep can advance
-constexpr int kStripMin = 96;           // smallest extent of a grid whose boundary strips run in the sweep's kernel
+constexpr int kStripMin = 96;           // smallest extent of a grid whose sweeps may have boundary strips
 constexpr int kStripCols = 4;           // columns of the left strip: one 16-byte group
 constexpr int kStripRow = 12;           // floats per row of a strip weight table (2R+1 weights, 16-byte rows)
 constexpr int kBopCopies = 16;          // most copies of the banded operands in global memory
@@ -893,16 +893,13 @@ bool strips_in_kernel(const MxRequest& q) {
     return fp32_class(q.prec) && q.n[0] >= kStripMin && q.n[1] >= kStripMin;
 }
 
-// Time steps per sweep.  k steps of an order-r stencil are one step of an
-// order-kr stencil, and the sweep's time grows far slower than k: 8192^2 TF32x3,
-// us per sweep for order 1 / 2 / 3 / 4: 89 / 94 / 113 / 125, so as many steps
-// as the largest order built (4) holds: 4 steps of order 1 in 125 us instead
-// of 356, 2 of order 2 instead of 188.  Only when the composed weights are as
-// safe as the single steps: within FP32's range by a wide margin, and with no
-// larger a rounding error (the composed weights' absolute sum bounds it; k
-// single steps have k times the weights' absolute sum, times the growth of a
-// constant field).
-int fused_depth(const MxRequest& q) {
+// Most time steps that one sweep may advance.  k steps of an order-r stencil
+// are one step of an order-kr stencil, as long as the largest order built (4)
+// holds it.  Only when the composed weights are as safe as the single steps:
+// within FP32's range by a wide margin, and with no larger a rounding error
+// (the composed weights' absolute sum bounds it; k single steps have k times
+// the weights' absolute sum, times the growth of a constant field).
+int most_depth(const MxRequest& q) {
     if (q.tb != 0 || !strips_in_kernel(q)) return 1;
     const int w = 2 * q.r + 1;
     double sum = 0.0, abs_sum = 0.0;
@@ -917,6 +914,80 @@ int fused_depth(const MxRequest& q) {
         if (composed <= 1.0001 * k * abs_sum * std::max(1.0, std::pow(std::fabs(sum), k - 1))) return k;
     }
     return 1;
+}
+
+// Grid region of the tiles of a sweep with strips of `rows` points along each
+// face (0: none), from an even row (row-parity views) and a 16-byte column
+// group, and the strip items: of whole rows, and beside the region.
+struct Region {
+    int x0 = 0, y0 = 0, x1, y1;
+    int64_t row_items = 0, col_items = 0;
+    Region(int ny, int nx, int rows) : x1(nx), y1(ny) {
+        if (rows <= 0) return;
+        x0 = kStripCols;
+        y0 = (rows + 1) / 2 * 2;
+        x1 = (nx - rows) / 4 * 4;
+        y1 = ny - rows;
+        const int groups = (nx + 3) / 4;
+        row_items = (int64_t)(y0 + ny - y1) * groups;
+        col_items = (int64_t)(y1 - y0) * (x0 / 4 + groups - x1 / 4);
+    }
+    int64_t items() const { return row_items + col_items; }
+};
+
+int strip_rows(int r, int bc, int depth) { return bc == kBcPeriodic ? depth * r : (depth - 1) * r; }
+
+// Estimated us per time step of sweeps of `depth` steps, with the faces as
+// strips in the sweep's kernel or (depth 1) as the periodic edge kernel's.  A
+// sweep's time grows far slower than its order: us per tile of an SM 1.5 / 1.6
+// / 1.8 / 2.05 for orders 1 to 4 (8192^2: 89 / 94 / 113 / 125), so many steps at
+// once are the faster, unless the strips outlast the tiles: one warp per CTA
+// takes about 4 us for 32 items along a row and 7 for 32 down a column
+// (periodic: 3.5 and 5.5), and short or narrow grids have many for their size.
+// The edge kernel takes a few us and some time per point, more down columns.
+// us per step, the rule's choice / the other: 1000000 x 96 r = 2 zero halo single
+// sweeps 124 / two steps with strips 1393; 96 x 1000000 r = 3 periodic edge kernel
+// 544 / strips 1242; 8192^2 r = 2 two steps with strips 66 / single sweeps 96.
+double step_cost(const MxRequest& q, int num_sms, int depth, bool strips) {
+    static const double kTile[5] = {0.0, 1.5, 1.6, 1.8, 2.05};
+    static const double kEdge[5] = {0.0, 2.5, 4.0, 6.0, 9.0};
+    static const double kEdgeRow[5] = {0.0, 15e-6, 23e-6, 40e-6, 60e-6};   // per point of whole rows
+    static const double kEdgeCol[5] = {0.0, 58e-6, 50e-6, 90e-6, 145e-6};  // per point down columns
+    const bool periodic = q.bc == kBcPeriodic;
+    const int ny = (int)q.n[0], nx = (int)q.n[1];
+    const Region g(ny, nx, strips ? strip_rows(q.r, q.bc, depth) : 0);
+    const int64_t tiles = tiles_2d(g.y1 - g.y0, g.x1 - g.x0, depth * q.r);
+    const int64_t ctas = std::min<int64_t>(num_sms, std::max<int64_t>(tiles, (g.items() + 31) / 32));
+    const double tile_us = (double)((tiles + ctas - 1) / ctas) * kTile[depth * q.r];
+    double strip_us = 0.0;
+    if (g.items() > 0) {
+        const double us = ((periodic ? 3.5 : 4.0) * g.row_items + (periodic ? 5.5 : 7.0) * g.col_items) / g.items();
+        strip_us = us * std::max(1.0, (double)g.items() / (32.0 * ctas));
+    }
+    const double edge_us =
+        periodic && !strips ? kEdge[q.r] + 2.0 * q.r * (ny * kEdgeCol[q.r] + nx * kEdgeRow[q.r]) : 0.0;
+    return (4.0 + std::max(tile_us, strip_us) + edge_us) / depth;
+}
+
+// Time steps per sweep, and whether its kernel computes the faces as strips.
+struct SweepKind {
+    int depth = 1;
+    bool strips = false;
+};
+
+SweepKind sweep_kind(const MxRequest& q, int num_sms) {
+    SweepKind best;
+    double least = step_cost(q, num_sms, 1, false);
+    const int deepest = most_depth(q);
+    for (int depth : {1, deepest}) {
+        if (!strips_in_kernel(q) || strip_rows(q.r, q.bc, depth) == 0) continue;
+        const double us = step_cost(q, num_sms, depth, true);
+        if (us < least) {
+            least = us;
+            best = {depth, true};
+        }
+    }
+    return best;
 }
 
 // Strip weights of depth k: [y class][x class][2R+1][kStripRow], classes 0 ..
@@ -996,8 +1067,16 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
     }
     const bool bf = is_bf16(q.prec);
     const int W = bf ? window<true>(kNb) : window<false>(kNb);
+    int dev = 0, num_sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) {
+        if (why) *why = std::string("device: ") + cudaGetErrorString(e);
+        return STENCIL_ECUDA;
+    }
+    const SweepKind kind = sweep_kind(q, num_sms);
     p->nb = kNb;
-    p->tb = fused_depth(q);
+    p->tb = kind.depth;
     p->n_lines = 2 * q.r + 1;
     p->cover = STENCIL_COVER_PARALLEL;
     p->n_scalar = 0;
@@ -1006,11 +1085,10 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
     // (CTA b reads copy b % copies).
     DepthOps depth[kMaxDepth + 1];
     std::vector<unsigned char> all(kSchedBytes, 0);
-    const bool strips = strips_in_kernel(q);
     for (int k = 1; k <= p->tb; ++k) {
         DepthOps& d = depth[k];
         d.order = k * q.r;
-        d.strip_rows = !strips ? 0 : q.bc == kBcPeriodic ? d.order : (k - 1) * q.r;
+        d.strip_rows = kind.strips ? strip_rows(q.r, q.bc, k) : 0;
         if (d.strip_rows > 0) {
             const int s = q.bc == kBcPeriodic ? 0 : d.strip_rows;
             const std::vector<float> w = strip_weights(q.r, q.cg, k, s);
@@ -1031,13 +1109,10 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
         all.insert(all.end(), ops.begin(), ops.end());
     }
     DepthOps& last = depth[p->tb];
-    int dev = 0, num_sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ctas = std::min<int64_t>(num_sms, tiles_2d(q.n[0], q.n[1], last.order));
     last.copies = (int)std::min<int64_t>(kBopCopies, (ctas + kCtasPerCopy - 1) / kCtasPerCopy);
     p->operand_bytes = all.size() + (size_t)(last.copies - 1) * last.bop_bytes;
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_operands, p->operand_bytes);
+    e = cudaMalloc(&p->d_operands, p->operand_bytes);
     if (e != cudaSuccess) {
         p->d_operands = nullptr;
         if (why) *why = std::string("operand upload: ") + cudaGetErrorString(e);
@@ -1083,7 +1158,7 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
         if (why) *why = std::string("kernel set-up: ") + cudaGetErrorString(e);
         return STENCIL_ECUDA;
     }
-    return strips ? STENCIL_OK : with_edges(q, p, why);   // the strips cover the periodic boundary
+    return kind.strips ? STENCIL_OK : with_edges(q, p, why);   // the strips cover the periodic boundary
 }
 
 void mx_plan_free(MxPlan* p) {
@@ -1137,20 +1212,15 @@ cudaError_t mx2d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
     a.bc = p.bc;
     a.in = (const float*)src;
     a.out = (float*)dst;
-    // The tiles' region: all of the grid, or what the strips leave, from an even
-    // row (row-parity views) and a whole 32-byte sector.
-    a.x1 = nx;
-    a.y1 = ny;
-    int64_t items = 0;
+    // the tiles' region: all of the grid, or what the strips leave
+    const Region region(ny, nx, d.strip_rows);
+    a.x0 = region.x0;
+    a.y0 = region.y0;
+    a.x1 = region.x1;
+    a.y1 = region.y1;
     if (d.strip_rows > 0) {
         a.strip_classes = d.strip_classes;
         a.strip_w = (const float*)((const unsigned char*)p.d_operands + d.strip_w);
-        a.x0 = kStripCols;
-        a.y0 = (d.strip_rows + 1) / 2 * 2;
-        a.x1 = (nx - d.strip_rows) / 4 * 4;
-        a.y1 = ny - d.strip_rows;
-        const int groups = (nx + 3) / 4;
-        items = (int64_t)(a.y0 + ny - a.y1) * groups + (int64_t)(a.y1 - a.y0) * (a.x0 / 4 + groups - a.x1 / 4);
     }
     const int rx = a.x1 - a.x0, ry = a.y1 - a.y0;
     a.tiles_x = (rx + kTw - 1) / kTw;
@@ -1172,7 +1242,7 @@ cudaError_t mx2d_sweep(const MxPlan& p, const void* src, void* dst, int tb, cuda
         return cudaErrorInvalidValue;
     const KernelInfo ki = kernel_for(d.order, st->bf, operand_parts(p.prec));
     // a CTA per tile or per warp of strip items, up to one per SM
-    const int64_t want = std::max<int64_t>(a.tiles_total, (items + 31) / 32);
+    const int64_t want = std::max<int64_t>(a.tiles_total, (region.items() + 31) / 32);
     const int grid = (int)std::min<int64_t>(want, st->num_sms);
     return launch_dependent(ki.fn, grid, kThreads, ki.smem, s, te, to, oe, oo, a);
 }
