@@ -872,12 +872,12 @@ std::vector<double> compose_steps(int r, const double* cg, int k, const Limits& 
             for (int x = -h; x <= h; ++x) {
                 const double v = cur[(size_t)(y + R) * W + x + R];
                 if (v == 0.0) continue;
-                for (int a = 0; a < w; ++a)
-                    for (int b = 0; b < w; ++b) {
-                        const int yy = y + a - r, xx = x + b - r;
-                        if (yy < in.ylo || yy > in.yhi || xx < in.xlo || xx > in.xhi) continue;
-                        nxt[(size_t)(yy + R) * W + xx + R] += cg[a * w + b] * v;
-                    }
+                const int a0 = std::max(0, in.ylo - y + r), a1 = std::min(w - 1, in.yhi - y + r);
+                const int b0 = std::max(0, in.xlo - x + r), b1 = std::min(w - 1, in.xhi - x + r);
+                for (int a = a0; a <= a1; ++a) {
+                    double* const row = &nxt[(size_t)(y + a - r + R) * W + x - r + R];
+                    for (int b = b0; b <= b1; ++b) row[b] += cg[a * w + b] * v;
+                }
             }
         cur.swap(nxt);
     }
@@ -1097,8 +1097,10 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
             all.insert(all.end(), (const unsigned char*)w.data(), (const unsigned char*)(w.data() + w.size()));
         }
         const std::vector<double> cg = compose_steps(q.r, q.cg, k, {-kNoLimit, kNoLimit, -kNoLimit, kNoLimit});
-        const std::vector<unsigned char> ops = pack_blocks(d.order, pair_blocks(d.order, cg.data()), kNb, W, bf,
-                                                           q.prec == STENCIL_PREC_TF32X3 && p->tb > 1, &d.bpart_bytes);
+        const bool cancel = q.prec == STENCIL_PREC_TF32X3 && p->tb > 1;
+        const std::vector<PairBlock> blocks = pair_blocks(d.order, cg.data());
+        const std::vector<unsigned char> ops = bf ? pack_blocks<true>(d.order, blocks, kNb, W, cancel, &d.bpart_bytes)
+                                                  : pack_blocks<false>(d.order, blocks, kNb, W, cancel, &d.bpart_bytes);
         d.bop_bytes = (uint32_t)ops.size();
         if (!kernel_for(d.order, bf, operand_parts(q.prec)).fn || d.bop_bytes != (bf ? 3 : 2) * d.bpart_bytes ||
             d.bop_bytes % 16 != 0) {

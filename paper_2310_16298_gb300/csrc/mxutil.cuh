@@ -303,14 +303,16 @@ struct PairBlock {
 // 2.9e-6..5.1e-6 without and 8.4e-8..6.1e-7 with.
 // Weights that are all exact in TF32 stay as they are: their products with
 // short mantissas are exact, and nothing is truncated.
-constexpr double kTrunc = 0.7213475 * 0.5 / (1 << 23);   // E[2^e / x] / 2 ulp, x's mantissa log-uniform
+constexpr double kUlp = 1.0 / (1 << 23);
+constexpr double kTrunc = 0.7213475 * 0.5 * kUlp;   // E[2^e / x] / 2 ulp, x's mantissa log-uniform
 
-inline std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& blocks, int nb, int kh,
-                                              bool bf, bool cancel, uint32_t* part_bytes) {
+template <bool bf>
+std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& blocks, int nb, int kh, bool cancel,
+                                       uint32_t* part_bytes) {
     const int nblk = (int)blocks.size(), N = nblk * nb, kw = 2 * kh;
-    const int epc = bf ? 8 : 4;  // elements per 16-byte chunk
-    const int es = bf ? 2 : 4;
-    const int parts = bf ? 3 : 2;
+    constexpr int epc = bf ? 8 : 4;  // elements per 16-byte chunk
+    constexpr int es = bf ? 2 : 4;
+    constexpr int parts = bf ? 3 : 2;
     const size_t pb = (size_t)(kw / epc) * N * 16;
     std::vector<unsigned char> out(parts * pb, 0);
     bool exact = true;
@@ -319,38 +321,43 @@ inline std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock
             for (int t = 0; b.line[e] && t < 2 * r + 1; ++t)
                 exact = exact && (double)tf32_round((float)b.line[e][t]) == b.line[e][t];
     cancel = cancel && !exact;
+    // The columns of a block are independent: they are packed side by side,
+    // weight by weight (one after the other, each is a chain of roundings).
     std::vector<double> carries(2 * nb, 0.0);      // per output parity and column
+    std::vector<int> adds(nb), step(nb);
     for (int j = 0; j < nblk; ++j) {
-        for (int q = 0; q < nb; ++q) {
-            double& carry = carries[blocks[j].parity * nb + q];
-            // band entry of line e at window column kk: weight kk - q - (4 - r)
-            auto weight = [&](int e, int kk) {
-                const int t = kk - q - (4 - r);
-                return blocks[j].line[e] && t >= 0 && t <= 2 * r ? blocks[j].line[e][t] : 0.0;
-            };
-            int adds = 0;                          // MMAs (8 columns each) that add to this block's column
-            if (cancel)
-                for (int e = 0; e < 2; ++e)
-                    for (int k0 = 0; k0 < kh; k0 += 8) {
-                        bool any = false;
-                        for (int kk = k0; kk < k0 + 8; ++kk) any = any || weight(e, kk) != 0.0;
-                        adds += any;
-                    }
-            for (int e = 0; e < 2; ++e) {
-                int step = -1;                     // last K step of this row that was counted
-                for (int kk = 0; kk < nb + 8; ++kk) {
-                    const double w = weight(e, kk);
-                    if (w == 0.0) continue;
+        double* const carry = &carries[blocks[j].parity * nb];
+        // adds[q]: MMAs (8 window columns each) that add to this block's column q;
+        // weight t of a line stands at window column q + 4 - r + t
+        std::fill(adds.begin(), adds.end(), 0);
+        for (int e = 0; e < 2; ++e) {
+            std::fill(step.begin(), step.end(), -1);
+            for (int t = 0; blocks[j].line[e] && t < 2 * r + 1; ++t) {
+                if (blocks[j].line[e][t] == 0.0) continue;
+                for (int q = 0; q < nb; ++q) {
+                    const int s = (q + 4 - r + t) / 8;
+                    adds[q] += step[q] != s;
+                    step[q] = s;
+                }
+            }
+        }
+        for (int e = 0; e < 2; ++e) {
+            std::fill(step.begin(), step.end(), -1);   // last K step of this row that was counted
+            for (int t = 0; blocks[j].line[e] && t < 2 * r + 1; ++t) {
+                const double w = blocks[j].line[e][t];
+                if (w == 0.0) continue;
+                const double most = std::fabs(w) * kUlp;
+                for (int q = 0; q < nb; ++q) {
+                    const int kk = q + 4 - r + t;
                     double rem = (double)(float)w;
                     if (cancel) {
-                        if (step >= 0 && step != kk / 8) --adds;
-                        step = kk / 8;
-                        const double most = std::ldexp(std::fabs(w), -23);
-                        const double taken = std::min(std::max(carry, -most), most);
-                        rem = w * (1.0 + (adds - 0.5) * kTrunc) + taken;
-                        carry -= taken;
+                        adds[q] -= step[q] >= 0 && step[q] != kk / 8;
+                        step[q] = kk / 8;
+                        const double taken = std::min(std::max(carry[q], -most), most);
+                        rem = w * (1.0 + (adds[q] - 0.5) * kTrunc) + taken;
+                        carry[q] -= taken;
                     }
-                    const int k = e * kh + kk;
+                    const unsigned k = e * kh + kk;
                     const size_t off = ((size_t)(k / epc) * N + (size_t)(j * nb + q)) * 16 + (size_t)(k % epc) * es;
                     for (int p = 0; p < parts; ++p) {
                         const float v = bf ? bf16_round((float)rem) : tf32_round((float)rem);
@@ -364,10 +371,10 @@ inline std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock
                             memcpy(&out[p * pb + off], &v, 4);
                         }
                     }
-                    if (cancel) carry += rem;
+                    if (cancel) carry[q] += rem;
                 }
-                if (step >= 0) --adds;
             }
+            for (int q = 0; q < nb; ++q) adds[q] -= step[q] >= 0;
         }
     }
     *part_bytes = (uint32_t)pb;
