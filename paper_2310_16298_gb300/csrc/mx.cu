@@ -102,6 +102,7 @@ constexpr int kStripCols = 4;           // columns of the left strip: one 16-byt
 constexpr int kStripRow = 12;           // floats per row of a strip weight table (2R+1 weights, 16-byte rows)
 constexpr int kBopCopies = 16;          // most copies of the banded operands in global memory
 constexpr int kCtasPerCopy = 10;        // CTAs that read one copy when a sweep starts
+constexpr size_t kMostOperands = (size_t)1 << 20;   // bytes of a plan's operands (what a server charges for them)
 constexpr int kMaxRawStages = 6;
 constexpr int kTileRing = 8;            // tile ids handed from the producer to the epilogue
 constexpr int kTmemCols = 512;
@@ -1113,6 +1114,7 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
     DepthOps& last = depth[p->tb];
     const int64_t ctas = std::min<int64_t>(num_sms, tiles_2d(q.n[0], q.n[1], last.order));
     last.copies = (int)std::min<int64_t>(kBopCopies, (ctas + kCtasPerCopy - 1) / kCtasPerCopy);
+    last.copies = (int)std::min<int64_t>(last.copies, 1 + (int64_t)(kMostOperands - all.size()) / last.bop_bytes);
     p->operand_bytes = all.size() + (size_t)(last.copies - 1) * last.bop_bytes;
     e = cudaMalloc(&p->d_operands, p->operand_bytes);
     if (e != cudaSuccess) {
