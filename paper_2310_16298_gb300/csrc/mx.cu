@@ -1098,7 +1098,7 @@ stencil_status mx_plan_build(const MxRequest& q, MxPlan* p, std::string* why) {
             all.insert(all.end(), (const unsigned char*)w.data(), (const unsigned char*)(w.data() + w.size()));
         }
         const std::vector<double> cg = compose_steps(q.r, q.cg, k, {-kNoLimit, kNoLimit, -kNoLimit, kNoLimit});
-        const bool cancel = q.prec == STENCIL_PREC_TF32X3 && p->tb > 1;
+        const bool cancel = p->tb > 1;
         const std::vector<PairBlock> blocks = pair_blocks(d.order, cg.data());
         const std::vector<unsigned char> ops = bf ? pack_blocks<true>(d.order, blocks, kNb, W, cancel, &d.bpart_bytes)
                                                   : pack_blocks<false>(d.order, blocks, kNb, W, cancel, &d.bpart_bytes);

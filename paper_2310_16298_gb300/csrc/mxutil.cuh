@@ -284,25 +284,36 @@ struct PairBlock {
 // first line (K rows 0 .. kh-1) over the band of its second (rows kh ..
 // 2kh-1).  Used when one TMEM lane holds two input rows side by side along K.
 //
-// `cancel` (fused TF32x3 sweeps): the error of TF32x3 over many steps is a bias
-// of the field's amplitude from two sources, both cancelled here at no cost (a
-// composed stencil's sums are longer, so its truncation is larger per sweep).
-//  * The low parts' rounding changes the weights' sum by up to 2^-24 of it:
-//    each output column's rounding errors are carried into its next weights
-//    (by at most 2^-23 of any weight, so that none is off by more than it
-//    would be rounded to FP32).
+// `cancel` (fused TF32x3 and BF16x3 sweeps): the error of these over many steps
+// is a bias of the field's amplitude from two sources, both cancelled here at
+// no cost (a composed stencil's sums are longer, so its truncation is larger per
+// sweep).
+//  * The last parts' rounding changes the weights' sum by up to 2^-24 of it:
+//    each output column's rounding errors are carried into its next weights,
+//    by at most 2^-23 of any weight.
 //  * The tensor core truncates an FP32 accumulator at each MMA that adds to
 //    it.  On average over mantissas that loses kTrunc of the accumulator's
 //    value, so a weight applied in the t-th last adding MMA of its block loses
 //    about t kTrunc of its product and is packed that much larger; by
-//    measurement (t - 1/2) kTrunc, for every order (the first MMA, on to the
-//    small correction products, loses less).
-// Relative L2 error after 100 steps over 10 random stencils (256 x 260,
-// positive field): order 1, single steps 1.8e-7..8.3e-6, fused by four 2.0e-6..3.1e-6
-// without and 1.2e-7..7.9e-7 with; order 2, single 1.3e-6..7.8e-6, fused by two
-// 2.9e-6..5.1e-6 without and 8.4e-8..6.1e-7 with.
-// Weights that are all exact in TF32 stay as they are: their products with
-// short mantissas are exact, and nothing is truncated.
+//    measurement (t - 1/2) kTrunc in TF32x3 and (t - 1) kTrunc in BF16x3, whose
+//    MMAs take twice the columns, for every order (the first MMA, on to the
+//    small correction products, loses less).  With up to six adding MMAs that
+//    is 2.4e-7 of a weight.
+// Products of either sign are corrected as if they had the accumulator's:
+// measured on signed weights and fields it helps there too.  Relative L2 error
+// after 100 steps, single steps / fused without / fused with (256 x 260, zero
+// halo and periodic, positive and signed fields):
+//   random weights, positive and signed, TF32x3: r = 1 1.2e-6..1.0e-5 single,
+//   9.7e-8..8.5e-7 fused with; r = 2 2.0e-6..7.6e-6, 7.8e-8..8.8e-7;
+//   BF16x3: r = 1 3.2e-6..4.8e-6 / 8.2e-7..1.7e-6 / 8.2e-8..6.1e-7, r = 2
+//   3.4e-6..5.1e-6 / 1.5e-6..2.6e-6 / 8.6e-8..7.5e-7;
+//   fourth-order diffusion (r = 2, weights of both signs), BF16x3
+//   2.0e-6..2.7e-6 / 2.7e-6..2.8e-6 / 5.7e-7..7.1e-7.
+// Weights that are all exact in one part stay as they are: fields of short
+// mantissas then have exact products and sums, which truncation leaves alone.
+// (Other fields' sums are truncated with such weights too, fused ones less
+// often per step: five-point smoothing with 1/2 and 1/8, single / fused, TF32x3
+// 2.3e-6..3.2e-6 / 1.0e-6..1.1e-6, BF16x3 2.4e-6..3.3e-6 / 9.9e-7..1.1e-6.)
 constexpr double kUlp = 1.0 / (1 << 23);
 constexpr double kTrunc = 0.7213475 * 0.5 * kUlp;   // E[2^e / x] / 2 ulp, x's mantissa log-uniform
 
@@ -313,13 +324,16 @@ std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& bloc
     constexpr int epc = bf ? 8 : 4;  // elements per 16-byte chunk
     constexpr int es = bf ? 2 : 4;
     constexpr int parts = bf ? 3 : 2;
+    constexpr int kstep = OpFmt<bf>::kKStep;
+    constexpr double first = bf ? 1.0 : 0.5;   // what the first MMA spares
     const size_t pb = (size_t)(kw / epc) * N * 16;
     std::vector<unsigned char> out(parts * pb, 0);
     bool exact = true;
     for (const auto& b : blocks)
         for (int e = 0; e < 2; ++e)
             for (int t = 0; b.line[e] && t < 2 * r + 1; ++t)
-                exact = exact && (double)tf32_round((float)b.line[e][t]) == b.line[e][t];
+                exact = exact && (double)(bf ? bf16_round((float)b.line[e][t]) : tf32_round((float)b.line[e][t])) ==
+                                     b.line[e][t];
     cancel = cancel && !exact;
     // The columns of a block are independent: they are packed side by side,
     // weight by weight (one after the other, each is a chain of roundings).
@@ -327,7 +341,7 @@ std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& bloc
     std::vector<int> adds(nb), step(nb);
     for (int j = 0; j < nblk; ++j) {
         double* const carry = &carries[blocks[j].parity * nb];
-        // adds[q]: MMAs (8 window columns each) that add to this block's column q;
+        // adds[q]: MMAs (kstep window columns each) that add to this block's column q;
         // weight t of a line stands at window column q + 4 - r + t
         std::fill(adds.begin(), adds.end(), 0);
         for (int e = 0; e < 2; ++e) {
@@ -335,7 +349,7 @@ std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& bloc
             for (int t = 0; blocks[j].line[e] && t < 2 * r + 1; ++t) {
                 if (blocks[j].line[e][t] == 0.0) continue;
                 for (int q = 0; q < nb; ++q) {
-                    const int s = (q + 4 - r + t) / 8;
+                    const int s = (q + 4 - r + t) / kstep;
                     adds[q] += step[q] != s;
                     step[q] = s;
                 }
@@ -351,10 +365,10 @@ std::vector<unsigned char> pack_blocks(int r, const std::vector<PairBlock>& bloc
                     const int kk = q + 4 - r + t;
                     double rem = (double)(float)w;
                     if (cancel) {
-                        adds[q] -= step[q] >= 0 && step[q] != kk / 8;
-                        step[q] = kk / 8;
+                        adds[q] -= step[q] >= 0 && step[q] != kk / kstep;
+                        step[q] = kk / kstep;
                         const double taken = std::min(std::max(carry[q], -most), most);
-                        rem = w * (1.0 + (adds[q] - 0.5) * kTrunc) + taken;
+                        rem = w * (1.0 + (adds[q] - first) * kTrunc) + taken;
                         carry[q] -= taken;
                     }
                     const unsigned k = e * kh + kk;
