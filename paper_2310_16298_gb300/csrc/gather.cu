@@ -891,8 +891,9 @@ gather3d_stream_kernel(const __grid_constant__ CUtensorMap tin, const G3Args a, 
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&tin);
     }
-    // as in the 2D kernel
-    if (sizeof(T) == 4 && (int)gridDim.x == a.units) ptx::launch_dependents();
+    // No early trigger of the next sweep, as in 2D: its CTAs would crowd on to the
+    // SMs with free slots and then share them while others idle (us per sweep
+    // with / without, r = 3 box 256^3 568 / 357, r = 1 box 256^3 76 / 54, 64^3 4.3 / 3.9).
     ptx::grid_dependency_wait();
     __syncthreads();
     int uses[NPL];   // TMA loads into each plane buffer so far (mbarrier phases)
