@@ -535,12 +535,20 @@ __device__ __forceinline__ bool gwait(uint64_t* bar, uint32_t parity) {
 // take 16 x 32 tiles (strips of 4 rows).  us per sweep before / after, star
 // r = 1: 256^2 8.3 / 2.8, 4096^2 187 / 175; box r = 2 4096^2 840 / 818, which is the
 // rate of bare FP64 FMAs on all SMs (510 G per second).
+// Several FP64 steps per sweep compute a halo of r (tb - t) points around the
+// tile at sub-step t, so grids with many tiles take 64 x 32 outputs by CTAs of
+// eight warps, two per SM (stars and r = 4 only while two fit the shared memory):
+// 4096^2, us per step with 32 / 64 rows, r = 3 star tb = 2 811 / 725, tb = 3
+// 994 / 868, r = 3 box tb = 3 3499 / 3204, tb = 4 (one CTA) 4081 / 3815, r = 2 box
+// tb = 4 1847 / 1709, r = 1 box tb = 4 628 / 615; one CTA: r = 4 star tb = 3
+// 1261 / 1357, box 100 x 30000 1370 / 1424.
 template <typename T>
 struct Tile2 {
     static constexpr int TY = 32;
     static constexpr int TYS = sizeof(T) == 4 ? 32 : 16;   // small grids
+    static constexpr int TYD = sizeof(T) == 4 ? 32 : 64;   // several steps per sweep, many tiles
     static constexpr int TX = sizeof(T) == 4 ? 128 : 32;
-    static constexpr int BY = sizeof(T) == 4 ? 8 : 4;
+    static constexpr int by(int ty) { return sizeof(T) == 4 || ty == 64 ? 8 : 4; }   // warps per CTA
     static constexpr int AL = 16 / (int)sizeof(T);   // TMA x granule (16 bytes)
 };
 __host__ __device__ constexpr int stages2(size_t elem, bool multi) { return elem == 4 && !multi ? 3 : 2; }
@@ -582,13 +590,13 @@ __device__ __forceinline__ void substep2(const T* src, T* dst, T* __restrict__ o
                                          bool last, int64_t ny, int64_t nx, int64_t ldx, int bc, int64_t y0, int64_t x0,
                                          const Coeffs<T, ipow(2 * R + 1, 2)>& cf) {
     constexpr int W = 2 * R + 1;
-    constexpr int RS = TY / Tile2<T>::BY;   // rows per strip
+    constexpr int RS = TY / Tile2<T>::by(TY);   // rows per strip
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int lo = R * t;                  // rows of the valid region skipped at the top
     const int lox = L.HX - L.H + R * t;    // columns skipped at the left
     const int Ht = L.SY - 2 * lo, Wt = L.SX - 2 * lox;
     const int nstrips = (Ht + RS - 1) / RS;
-    for (int strip = ty; strip < nstrips; strip += Tile2<T>::BY) {
+    for (int strip = ty; strip < nstrips; strip += Tile2<T>::by(TY)) {
         const int sy0 = lo + strip * RS;
         for (int c = tx; c < Wt; c += kBX) {
             const int sx = lox + c;
@@ -695,17 +703,17 @@ __device__ __noinline__ void wrap_halo_block(T* buf, int SY, int SX, const T* __
 
 // Register budgets of the persistent kernels: left alone, the compiler keeps
 // the coefficients and unrolled sums in registers and one CTA fills an SM.
-template <typename T, int R, bool STAR, bool MULTI>
+template <typename T, int R, bool STAR, bool MULTI, int TY>
 constexpr int ctas2() {
-    if (sizeof(T) == 8) return STAR && R >= 3 ? 2 : 4;   // (strips of wide stars hold 2r+1 rows in registers)
+    if (sizeof(T) == 8) return TY == 64 || (STAR && R >= 3) ? 2 : 4;   // (strips of wide stars hold 2r+1 rows in registers)
     return MULTI ? (R == 1 ? 3 : R == 2 ? 2 : 1) : (STAR && R >= 4) ? 2 : 3;
 }
 
 template <typename T, int R, bool STAR, bool MULTI, int TY>
-__global__ void __launch_bounds__(kBX * Tile2<T>::BY, (ctas2<T, R, STAR, MULTI>()))
+__global__ void __launch_bounds__(kBX * Tile2<T>::by(TY), (ctas2<T, R, STAR, MULTI, TY>()))
 gather2d_tma_kernel(const __grid_constant__ CUtensorMap tin, const G2Args a, const Coeffs<T, ipow(2 * R + 1, 2)> cf) {
     constexpr int TX = Tile2<T>::TX;
-    constexpr int kThr = kBX * Tile2<T>::BY;
+    constexpr int kThr = kBX * Tile2<T>::by(TY);
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char* smem_raw = (unsigned char*)(((uintptr_t)smem_dyn + 127) & ~(uintptr_t)127);
     const Layout2<T, TY> L(R, a.tb);
@@ -1159,24 +1167,30 @@ cudaError_t launch2d_tma(const GatherProblem& p, const void* in, void* out, int 
     if (!encode_grid_map<T>(&tin, in, 2, dims, p.ldx, box)) return cudaErrorInvalidValue;
     constexpr bool F32 = sizeof(T) == 4;
     auto kern = F32 && tb > 1 ? gather2d_tma_kernel<T, R, STAR, F32, TY> : gather2d_tma_kernel<T, R, STAR, false, TY>;
-    constexpr int threads = kBX * Tile2<T>::BY;
+    constexpr int threads = kBX * Tile2<T>::by(TY);
     GatherTuned t;
     cudaError_t e = tuned_for(p, kern, threads, smem, tb, &t);
     if (e != cudaSuccess || p.prepare) return e;
     int grid = t.sms * t.per_sm[tb];
     if (grid > a.tiles_total) grid = a.tiles_total;
     a.sched = sizeof(T) == 4 && grid < a.tiles_total ? p.sched : nullptr;   // FP64: compute-bound, fixed shares do
-    return launch_dependent(kern, dim3(grid), dim3(kBX, Tile2<T>::BY), smem, s, tin, a, cf);
+    return launch_dependent(kern, dim3(grid), dim3(kBX, Tile2<T>::by(TY)), smem, s, tin, a, cf);
 }
 
 template <typename T, int R, bool STAR>
 cudaError_t launch2d(const GatherProblem& p, const void* in, void* out, int tb, cudaStream_t s) {
-    constexpr int TY = Tile2<T>::TY, TYS = Tile2<T>::TYS, TX = Tile2<T>::TX;
+    constexpr int TY = Tile2<T>::TY, TYS = Tile2<T>::TYS, TYD = Tile2<T>::TYD, TX = Tile2<T>::TX;
     const Layout2<T, TY> L(R, tb);
     if (!tma_layout_ok<T>(p, in) || L.bytes(tb) > (size_t)smem_limit(p) || L.SX > 256 || L.SY > 256)
         return p.prepare ? cudaSuccess : launch2d_tiles<T, R, STAR>(p, in, out, tb, s);
-    const int64_t tiles = ((p.n[0] + TY - 1) / TY) * ((p.n[1] + TX - 1) / TX);
-    if (TYS != TY && tiles < (p.tuned ? p.tuned->sms : sm_count())) return launch2d_tma<T, R, STAR, TYS>(p, in, out, tb, s);
+    const int64_t tiles_x = (p.n[1] + TX - 1) / TX, tiles = ((p.n[0] + TY - 1) / TY) * tiles_x;
+    const int sms = p.tuned ? p.tuned->sms : sm_count();
+    if (TYD != TY && tb > 1 && (p.n[0] + TYD - 1) / TYD * tiles_x >= 8 * sms) {
+        const Layout2<T, TYD> D(R, tb);
+        if (D.bytes(tb) <= (size_t)smem_limit(p) / (STAR || R == 4 ? 2 : 1) && D.SY <= 256)
+            return launch2d_tma<T, R, STAR, TYD>(p, in, out, tb, s);
+    }
+    if (TYS != TY && tiles < sms) return launch2d_tma<T, R, STAR, TYS>(p, in, out, tb, s);
     return launch2d_tma<T, R, STAR, TY>(p, in, out, tb, s);
 }
 
