@@ -373,9 +373,10 @@ gather2d_kernel(const T* __restrict__ in, T* __restrict__ out, int64_t ny, int64
 // p owns tiles [tile0[p], tile0[p+1]); its coefficients sit at coef + p*NC.
 // Registers: FP64 two CTAs' worth per SM (with one, the compiler takes up to 254
 // and a lone CTA's barriers leave the FP64 pipe idle: 48 problems of up to 1500^2,
-// 24 steps, r = 1 star 3.89 ms, with two 3.22; r = 3 star 7.20 and 6.30).
+// 24 steps, r = 1 star 3.89 ms, with two 3.22; r = 3 star 7.20 and 6.30), but for
+// the 49 weights of r = 3 boxes in the large tile (22.6 ms, with two 25.3).
 template <typename T, int R, bool STAR, int BY, int TX, int TY>
-__global__ void __launch_bounds__(kBX * BY, sizeof(T) == 8 ? 2 : R == 1 ? 16 / BY + 1 : 1)
+__global__ void __launch_bounds__(kBX * BY, sizeof(T) == 8 ? (R == 3 && !STAR && TY == 64 ? 1 : 2) : R == 1 ? 16 / BY + 1 : 1)
 gather2d_batch_kernel(const BatchProblem* __restrict__ probs, int nprob, int total_tiles,
                       const T* __restrict__ coef) {
     constexpr int NC = ipow(2 * R + 1, 2);
