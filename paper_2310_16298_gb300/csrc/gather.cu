@@ -1226,9 +1226,12 @@ cudaError_t launch3d(const GatherProblem& p, const void* in, void* out, int tb, 
     int grid = t.sms * t.per_sm[1];
     // A unit's fixed cost in planes: FP32 units re-read 2R halo planes and wait
     // for the first 2R + 1 to land; FP64 units compute far longer than that per
-    // plane, so even shares matter most.
+    // plane, so even shares matter most.  Four FP64 CTAs on an SM run faster when
+    // two have nothing left; one alone of two (r >= 3) does not keep the FP64 pipe
+    // busy, so there whole waves count (256^3 r = 3 in half waves / whole: star
+    // 846 / 681 us per sweep, box 14637 / 11726).
     const int tiles = a.tiles_x * a.tiles_y;
-    a.tzc = sizeof(T) == 8 ? pick_chunk(a.nz, tiles, grid, 2, 1, 64, 1 << 20)
+    a.tzc = sizeof(T) == 8 ? pick_chunk(a.nz, tiles, grid, t.per_sm[1] >= 4 ? 2 : 1, 1, 64, 1 << 20)
                            : pick_chunk(a.nz, tiles, grid, 2, 2 * R + 2, 64, 32);
     a.units = tiles * ((a.nz + a.tzc - 1) / a.tzc);
     if (grid > a.units) grid = a.units;
