@@ -18,8 +18,8 @@
 // latency on the critical path of every edge tile, and slowed the 2D sweep by
 // up to a half and the 3D sweep up to fourfold; here the boundary costs one
 // short launch over about 2 r (nx + ny) nz points, one thread per point.  3D
-// plans use it, and 2D ones on small grids or in plain precisions; the other 2D
-// sweeps compute their strips beside the tiles (boundary_strips in mx.cu).
+// plans use it, and 2D ones on small, short or narrow grids or in plain
+// precisions; the other 2D sweeps compute their strips beside the tiles (boundary_strips in mx.cu).
 #include <cuda_runtime.h>
 #include <stdint.h>
 

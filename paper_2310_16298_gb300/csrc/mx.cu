@@ -36,8 +36,9 @@
 // fill (the zero Dirichlet halo).  With a periodic boundary, or when a sweep
 // advances several steps (R is then the order of the composed stencil), the
 // points near the faces are boundary strips, computed beside the tiles; on
-// small grids and in plain precisions the periodic boundary's wrapped terms
-// are added afterwards by the edge kernel (edges.cu).
+// small, short or narrow grids (sweep_kind) and in plain precisions the
+// periodic boundary's wrapped terms are added afterwards by the edge kernel
+// (edges.cu).
 //
 // Roles (one persistent CTA per SM, warp specialised):
 //  * warp 0: TMA producer.  A tile is 4 lane quarters x 64 input rows; each

@@ -95,8 +95,9 @@ struct stencil_server_s {
     // statistics
     int64_t admitted = 0, completed = 0, peak_resident = 0, peak_bytes = 0;
     std::atomic<int64_t> issued{0};
-    // Finished plans are destroyed in groups (freeing a plan's scratch grid
-    // synchronises the device); their memory stays charged until then.
+    // Finished plans are destroyed when the worker is idle, one at a time, or all
+    // at once when the budget needs their memory (freeing a plan's scratch grid
+    // synchronises the device); it stays charged until then.
     std::vector<std::pair<stencil_plan_t, int64_t>> graveyard;
     // Pinned result buffers that came back, by size, for later requests: pinning
     // and unpinning fresh memory took most of a burst's host time (24 requests,
