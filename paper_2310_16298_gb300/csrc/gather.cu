@@ -534,8 +534,8 @@ __device__ __forceinline__ bool gwait(uint64_t* bar, uint32_t parity) {
 // and SM) is the limit, and with two CTAs of eight warps it sat idle a quarter
 // of the time around their barriers.  Grids with fewer such tiles than SMs
 // take 16 x 32 tiles (strips of 4 rows).  us per sweep before / after, star
-// r = 1: 256^2 8.3 / 2.8, 4096^2 187 / 175; box r = 2 4096^2 840 / 818, which is the
-// rate of bare FP64 FMAs on all SMs (510 G per second).
+// r = 1: 256^2 8.3 / 2.8, 4096^2 187 / 175; box r = 2 4096^2 840 / 815: 515 G FMAs per
+// second, where bare FP64 FMAs on all SMs reach 525.
 // Several FP64 steps per sweep compute a halo of r (tb - t) points around the
 // tile at sub-step t, so grids with many tiles take 64 x 32 outputs by CTAs of
 // eight warps, two per SM (stars and r = 4 only while two fit the shared memory):
