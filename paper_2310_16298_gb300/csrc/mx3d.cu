@@ -56,8 +56,9 @@ constexpr int kMaxRawStages = 6;
 constexpr int kUnitRing = 8;                // unit ids handed from the producer to the epilogue
 constexpr int kTmemCols = 512;
 constexpr int kSmemBudget = 227 * 1024;
-// Deepest work unit the library chooses (plans may set their own depth): at 512^3
-// 16 to 32 planes ran fastest, 64 and 128 slower (fewer units to balance).
+// Deepest work unit the library chooses (plans may set their own depth): us per
+// 512^3 sweep by planes per unit, 7-point 16 / 32 / 64 / 128 217 / 207 / 203 / 201,
+// 27-point 387 / 373 / 361 / 356; the depth chosen, by whole waves, 196 and 360.
 constexpr int kMaxChunk = 32;
 // Pipeline fill and drain of a unit, in plane times (pick_chunk's fixed cost beside the 2R halo planes).
 constexpr int kFillPlanes = 2;
